@@ -19,11 +19,10 @@ template <class S, int LAYOUT>
 cudaError_t step_layout(const BoxStep<S> &b, bool noise, bool force, dim3 grid, dim3 block, const uint32_t *p,
                         uint32_t t, cudaStream_t st)
 {
-    if (noise && force) k_stream_collide<S, LAYOUT, true, true><<<grid, block, 0, st>>>(b, p, t);
-    else if (noise) k_stream_collide<S, LAYOUT, true, false><<<grid, block, 0, st>>>(b, p, t);
-    else if (force) k_stream_collide<S, LAYOUT, false, true><<<grid, block, 0, st>>>(b, p, t);
-    else k_stream_collide<S, LAYOUT, false, false><<<grid, block, 0, st>>>(b, p, t);
-    return cudaGetLastError();
+    if (noise && force) return launch_chained(k_stream_collide<S, LAYOUT, true, true>, grid, block, st, b, p, t);
+    if (noise) return launch_chained(k_stream_collide<S, LAYOUT, true, false>, grid, block, st, b, p, t);
+    if (force) return launch_chained(k_stream_collide<S, LAYOUT, false, true>, grid, block, st, b, p, t);
+    return launch_chained(k_stream_collide<S, LAYOUT, false, false>, grid, block, st, b, p, t);
 }
 
 // V sites per thread: 16-byte accesses for 4-byte formats, 8-byte for 16-bit, V = 2 for FP64.
@@ -38,11 +37,10 @@ cudaError_t step_layout_vec(const BoxStep<S> &b, bool noise, bool force, dim3 gr
                             uint32_t t, cudaStream_t st)
 {
     constexpr int V = vec_width<S>();
-    if (noise && force) k_stream_collide_vec<S, LAYOUT, true, true, V><<<grid, block, 0, st>>>(b, p, t);
-    else if (noise) k_stream_collide_vec<S, LAYOUT, true, false, V><<<grid, block, 0, st>>>(b, p, t);
-    else if (force) k_stream_collide_vec<S, LAYOUT, false, true, V><<<grid, block, 0, st>>>(b, p, t);
-    else k_stream_collide_vec<S, LAYOUT, false, false, V><<<grid, block, 0, st>>>(b, p, t);
-    return cudaGetLastError();
+    if (noise && force) return launch_chained(k_stream_collide_vec<S, LAYOUT, true, true, V>, grid, block, st, b, p, t);
+    if (noise) return launch_chained(k_stream_collide_vec<S, LAYOUT, true, false, V>, grid, block, st, b, p, t);
+    if (force) return launch_chained(k_stream_collide_vec<S, LAYOUT, false, true, V>, grid, block, st, b, p, t);
+    return launch_chained(k_stream_collide_vec<S, LAYOUT, false, false, V>, grid, block, st, b, p, t);
 }
 
 }  // namespace

@@ -207,6 +207,7 @@ template <class S, int LAYOUT, bool NOISE, bool FORCE>
 __global__ void __launch_bounds__(256) k_stream_collide(const BoxStep<S> B, const uint32_t *step_ptr, uint32_t step)
 {
     using R = typename Storage<S>::R;
+    let_next_step_start();
     const int bxi = blockIdx.x % B.gx, byi = blockIdx.x / B.gx;
     const int x = bxi * blockDim.x + threadIdx.x;
     const int y = byi * blockDim.y + threadIdx.y;
@@ -220,6 +221,7 @@ __global__ void __launch_bounds__(256) k_stream_collide(const BoxStep<S> B, cons
     auto xpush = [&](int c) { return c > 0 ? xp : (c < 0 ? xm : x); };      // x + c
     auto ypush = [&](int c) { return c > 0 ? yp : (c < 0 ? ym : y); };
     const int site = y * nx + x;
+    wait_for_previous_step();
     R f[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -255,7 +257,7 @@ template <class S, int V>
 __device__ __forceinline__ void load_vec2(const S *p, S (&out)[V])
 {
     using T = typename RawVec2<sizeof(S) * V>::T;
-    const T raw = __ldg(reinterpret_cast<const T *>(p));
+    const T raw = *reinterpret_cast<const T *>(p);
     const S *e = reinterpret_cast<const S *>(&raw);
 #pragma unroll
     for (int v = 0; v < V; ++v) out[v] = e[v];
@@ -277,6 +279,7 @@ __global__ void __launch_bounds__(256, sizeof(typename Storage<S>::R) == 4 ? (si
 k_stream_collide_vec(const BoxStep<S> B, const uint32_t *step_ptr, uint32_t step)
 {
     using R = typename Storage<S>::R;
+    let_next_step_start();
     const int nx = B.nx, ny = B.ny, gx = nx / V;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int lane = tid & 31;
@@ -290,6 +293,7 @@ k_stream_collide_vec(const BoxStep<S> B, const uint32_t *step_ptr, uint32_t step
     const bool shr = lane < 31 && x0 + V != nx;       // lane + 1 owns x0 + V ..
     const int x_left = x0 == 0 ? nx - 1 : x0 - 1, x_right = x0 + V == nx ? 0 : x0 + V;
     const int x_lload = shl ? x0 : x_left, x_rload = shr ? x0 + V - 1 : x_right;
+    wait_for_previous_step();
     S raw[Q][V];
     S edge[Q];
 #pragma unroll

@@ -262,6 +262,22 @@ __device__ __forceinline__ void gaussians15(uint32_t site, uint32_t step, uint32
     }
 }
 
+// The normals that the collision of one site (R = F2: of two sites) uses.
+template <class R, class KR, class SiteT>
+__device__ __forceinline__ void draw_normals(const CollideConsts<KR> &K, SiteT site, uint32_t step, uint32_t replica,
+                                             R (&g)[16])
+{
+    if constexpr (std::is_same<R, F2>::value) {   // a pair of sites: each its own normals
+        float ga[16], gb[16];
+        gaussians15<float>(site.x, step, replica, K.rk0, K.rk1, bm_of(K), ga);
+        gaussians15<float>(site.y, step, replica, K.rk0, K.rk1, bm_of(K), gb);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) g[k] = R(ga[k], gb[k]);
+    } else {
+        gaussians15<R>(site, step, replica, K.rk0, K.rk1, bm_of(K), g);
+    }
+}
+
 // --------------------------------------------------------------------------
 // Forward transform m_k = sum_i e_ki f_i (Table II), on the pair sums s and
 // differences d of opposite velocities.
@@ -340,9 +356,11 @@ __device__ __forceinline__ void forward_modes(const R (&f)[Q], R (&m)[Q])
 // NOISE: 0 = deterministic, 1 = thermal noise, 2 = thermal noise with
 // gamma_ghost = 0 (the kinetic modes carry only their noise, so their forward
 // transform and relaxation are skipped).
-template <class R, int NOISE, bool FORCE, class KR, class SiteT>
+// DRAWN: g already holds the site's normals (draw_normals); otherwise they are
+// drawn here, after the forward transform.
+template <class R, int NOISE, bool FORCE, bool DRAWN, class KR, class SiteT>
 __device__ __forceinline__ void collide(R (&f)[Q], const CollideConsts<KR> &K, SiteT site, uint32_t step,
-                                        uint32_t replica, R Fx)
+                                        uint32_t replica, R Fx, R (&g)[16])
 {
     constexpr bool kin0 = NOISE == 2;
     R m[Q];
@@ -397,16 +415,7 @@ __device__ __forceinline__ void collide(R (&f)[Q], const CollideConsts<KR> &K, S
         t[9] += K.forcing[9] * (uz * Fx);
     }
     if (NOISE) {
-        R g[16];
-        if constexpr (std::is_same<R, F2>::value) {   // a pair of sites: each its own normals
-            float ga[16], gb[16];
-            gaussians15<float>(site.x, step, replica, K.rk0, K.rk1, bm_of(K), ga);
-            gaussians15<float>(site.y, step, replica, K.rk0, K.rk1, bm_of(K), gb);
-#pragma unroll
-            for (int k = 0; k < 16; ++k) g[k] = R(ga[k], gb[k]);
-        } else {
-            gaussians15<R>(site, step, replica, K.rk0, K.rk1, bm_of(K), g);
-        }
+        if constexpr (!DRAWN) draw_normals<R>(K, site, step, replica, g);
         if (K.noise_rho_local) {
             // variance mu rho w_k with the local density
             const R scale = sqrt_r(rho * K.inv_rho0);
@@ -559,16 +568,18 @@ struct Storage<bf16sr> {
     __device__ static double to_double(bf16sr v) { return (double)load(v); }
 };
 
-// Read-only cached load of one stored element (the 16-bit pattern for bf16sr).
+// Load of one stored element (the 16-bit pattern for bf16sr).  An ordinary
+// load: a step's kernel starts while the one before it still writes (see
+// wait_for_previous_step), which the read-only path does not allow.
 template <class S>
 __device__ __forceinline__ S load_ro(const S *p)
 {
-    return __ldg(p);
+    return *p;
 }
 template <>
 __device__ __forceinline__ bf16sr load_ro<bf16sr>(const bf16sr *p)
 {
-    return bf16sr{__ldg(reinterpret_cast<const unsigned short *>(p))};
+    return bf16sr{*reinterpret_cast<const unsigned short *>(p)};
 }
 
 // Stochastic rounding of x to bfloat16 with 16 random bits r: r is added to
@@ -639,6 +650,18 @@ __device__ __forceinline__ bool span_ok(const S *base, int64_t plane, const S *p
 #define FLB_GUARD_LD(B, p, n) (p)
 #define FLB_GUARD_ST(B, p, n) true
 #endif
+
+// --------------------------------------------------------------------------
+// Chained steps.  The step kernels are launched with programmatic stream
+// serialization: a step's blocks are scheduled as soon as every block of the
+// step before has started (let_next_step_start), and do what needs no stored
+// state -- index arithmetic, and in the small-box kernels the Gaussian numbers
+// -- before wait_for_previous_step, which returns when the whole step before has
+// finished and its writes are visible.  Every block of every step kernel
+// waits, so a finished step implies that all the steps before it have finished.
+// --------------------------------------------------------------------------
+__device__ __forceinline__ void let_next_step_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous_step() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // --------------------------------------------------------------------------
 // Where the canonical pre-collision population n_i(r, t) lives in device memory.

@@ -33,6 +33,25 @@ struct Launch {
     bool warprow = false;   // one box, bx * V == nx, bx divides 32: rows tile the warps, shuffles only
 };
 
+// Launches a step kernel with programmatic stream serialization: its blocks may
+// start once every block of the kernel before it has called
+// let_next_step_start (a kernel that never does is waited for as usual), and it
+// calls wait_for_previous_step before it touches the state.
+template <class... KA, class... A>
+cudaError_t launch_chained(void (*kernel)(KA...), dim3 grid, dim3 block, cudaStream_t st, const A &...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // The FP64 Box-Muller tables (BoxMullerTables): r[65536] then cs[65536] in one
 // allocation of kBoxMullerTableBytes, filled by one launch.
 constexpr size_t kBoxMullerTableBytes = 65536 * (sizeof(double) + sizeof(double2));

@@ -34,6 +34,21 @@ struct BoxStep {
     FLB_VIOL_FIELD
 };
 
+// When a step's blocks let the next step's blocks start (see d3q19.cuh).  Four
+// sites per thread, the launches of many waves: at their own start, so that the
+// next step fills the SMs that the last wave leaves.  Fewer sites per thread,
+// the boxes of a wave or less: once their loads are back -- any sooner and the
+// next step's blocks crowd onto the SMs that happen to be free, which unbalances
+// every later step.  FP64, whose collision keeps the SM's FP64 unit busy for
+// microseconds: before the stores.  Measured per step, plain launches, at the
+// start / after the loads / before the stores (8.20, 6.16, 4.11 and 10.3 us for
+// unchained launches): 64^3 FP32 6.26 / 6.02 / 5.94 us, 48^3 FP32 5.32 / 3.80 /
+// 4.03, 16^3 FP32 2.26 / 1.69 / 1.92, 16^3 FP64 8.26 / 8.06 / 7.84, 32^3 FP64
+// 39.9 / 16.6 / 16.1; V = 4: 96^3 FP32 28.8 / 29.8 / 29.1.
+enum StartPoint : int { kAtStart = 0, kAfterLoads = 1, kBeforeStores = 2 };
+template <class S, int V>
+constexpr StartPoint kStart = sizeof(S) == 8 ? kBeforeStores : (V >= 4 ? kAtStart : kAfterLoads);
+
 template <class S, int LAYOUT, int NOISE, bool FORCE, int V>
 __device__ __forceinline__ void update_sites(const BoxStep<S> &B, int x0, int y, int z, uint32_t step)
 {
@@ -50,11 +65,12 @@ __device__ __forceinline__ void update_sites(const BoxStep<S> &B, int x0, int y,
     R Fx = R(0);
     if (FORCE) Fx = B.K.force_amp * sin_pi(B.K.force_phase * R(z));
     const uint32_t site_row = (uint32_t)row(y, z);
-
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-        const int x = x0 + v;
-        if (x >= nx) break;
+    static_assert(V == 1, "the scalar path takes one site per thread");
+    {
+        const int x = x0;
+        R g[16];
+        if (NOISE) draw_normals<R>(B.K, site_row + (uint32_t)x, step, B.replica, g);
+        wait_for_previous_step();
         const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
         auto xsel = [&](int c) { return c > 0 ? xm : (c < 0 ? xp : x); };
         auto xsel_push = [&](int c) { return c > 0 ? xp : (c < 0 ? xm : x); };
@@ -72,8 +88,10 @@ __device__ __forceinline__ void update_sites(const BoxStep<S> &B, int x0, int y,
             const S *p = B.src + (int64_t)slot * B.plane + idx;
             f[i] = Storage<S>::load(load_ro(FLB_GUARD_LD(B, p, 1)));
         }
-        collide<R, NOISE, FORCE>(f, B.K, site_row + (uint32_t)x, step, B.replica, Fx);
+        if constexpr (kStart<S, V> == kAfterLoads) let_next_step_start();
+        collide<R, NOISE, FORCE, true>(f, B.K, site_row + (uint32_t)x, step, B.replica, Fx, g);
         stochastic_round<S>(f, site_row + (uint32_t)x, step, B.replica, B.K.rk0, B.K.rk1);
+        if constexpr (kStart<S, V> == kBeforeStores) let_next_step_start();
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             int idx, slot;
@@ -122,7 +140,7 @@ template <class S, int V>
 __device__ __forceinline__ void load_vec(const S *p, S (&out)[V])
 {
     using T = typename RawVec<sizeof(S) * V>::T;
-    const T raw = __ldg(reinterpret_cast<const T *>(p));
+    const T raw = *reinterpret_cast<const T *>(p);
     const S *e = reinterpret_cast<const S *>(&raw);
 #pragma unroll
     for (int v = 0; v < V; ++v) out[v] = e[v];
@@ -283,6 +301,24 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
     const int x_lload = shl ? x0 : x_left;
     const int x_rload = shr ? x0 + V - 1 : x_right;
 
+    const uint32_t site0 = (uint32_t)(zo[1] + yo[1]) + (uint32_t)x0;
+    // Two sites per thread in rows of whole warps (the small boxes): the normals,
+    // which need no stored state, before the wait; four sites' would not fit
+    // beside the populations, and a step of many waves runs 5 % slower with the
+    // loads behind them (250 x 187 x 93 FP32, 131 against 125 us).
+    constexpr bool kPaired = sizeof(R) == 4 && sizeof(S) == 2 && V % 2 == 0;
+    constexpr bool kDrawn = NOISE && V == 2 && WARPROW;
+    using G = typename std::conditional<kPaired, F2, R>::type;
+    constexpr int NG = kPaired ? V / 2 : V;
+    G g[kDrawn ? NG : 1][16];
+    if constexpr (kDrawn && kPaired) {
+        draw_normals<F2>(B.K, make_uint2(site0, site0 + 1), step, B.replica, g[0]);
+    } else if constexpr (kDrawn) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) draw_normals<R>(B.K, site0 + v, step, B.replica, g[v]);
+    }
+    wait_for_previous_step();
+
     // 1. issue every load of the 19 planes (vector + edge element) before
     //    any shuffle, so that all of them are in flight together
     S raw[Q][V];
@@ -354,18 +390,19 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
     }
 
     R Fx = R(0);
+    if constexpr (kStart<S, V> == kAfterLoads) let_next_step_start();
     if (FORCE) Fx = B.K.force_amp * sin_pi(B.K.force_phase * R(z));
-    const uint32_t site0 = (uint32_t)(zo[1] + yo[1]) + (uint32_t)x0;
     // 16-bit formats (issue-bound): two sites per collision in the paired FP32
     // instructions; FP32 storage is bound by HBM and keeps the one-site form,
     // whose odd AA step measured faster
-    if constexpr (sizeof(R) == 4 && sizeof(S) == 2 && V % 2 == 0) {
+    if constexpr (kPaired) {
 #pragma unroll
         for (int v = 0; v < V; v += 2) {
             F2 p[Q];
 #pragma unroll
             for (int i = 0; i < Q; ++i) p[i] = F2(f[v][i], f[v + 1][i]);
-            collide<F2, NOISE, FORCE>(p, B.K, make_uint2(site0 + v, site0 + v + 1), step, B.replica, F2(Fx));
+            collide<F2, NOISE, FORCE, kDrawn>(p, B.K, make_uint2(site0 + v, site0 + v + 1), step, B.replica, F2(Fx),
+                                              g[kDrawn ? v / 2 : 0]);
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 f[v][i] = p[i].v.x;
@@ -374,11 +411,13 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
         }
     } else {
 #pragma unroll
-        for (int v = 0; v < V; ++v) collide<R, NOISE, FORCE>(f[v], B.K, site0 + v, step, B.replica, Fx);
+        for (int v = 0; v < V; ++v)
+            collide<R, NOISE, FORCE, kDrawn>(f[v], B.K, site0 + v, step, B.replica, Fx, g[kDrawn ? v : 0]);
     }
 #pragma unroll
     for (int v = 0; v < V; ++v) stochastic_round<S>(f[v], site0 + v, step, B.replica, B.K.rk0, B.K.rk1);
 
+    if constexpr (kStart<S, V> == kBeforeStores) let_next_step_start();
     R pushed[Q];   // FULLROW, AA odd: the value crossing into this warp's vector from the neighbour warp
     if (FULLROW && LAYOUT == kAAOdd) {
 #pragma unroll
@@ -500,6 +539,7 @@ template <class S, int LAYOUT, int NOISE, bool FORCE, int V, bool FULLROW, bool 
 __device__ __forceinline__ void stream_collide_box(const BoxStep<S> &B, const uint32_t *step_ptr, uint32_t step)
 {
     static_assert(!UROW || FULLROW, "UROW is a FULLROW launch");
+    if constexpr (kStart<S, V> == kAtStart) let_next_step_start();
     int x0 = V * (blockIdx.x * blockDim.x + threadIdx.x);
     int y = UROW ? (int)blockIdx.y : (int)(blockIdx.y * blockDim.y + threadIdx.y);
     const int z = B.z0 + (int)blockIdx.z;
@@ -569,6 +609,7 @@ template <class S, int LAYOUT, int NOISE, bool FORCE, int V>
 __global__ void __launch_bounds__(256) k_stream_collide_batch(const __grid_constant__ BatchParams<S> P,
                                                               const uint32_t *step_ptr, uint32_t step)
 {
+    if constexpr (kStart<S, V> == kAtStart) let_next_step_start();
     // last box with block0 <= blockIdx.x (the same for the whole block)
     int lo = 0, hi = P.nboxes - 1;
     const int b = (int)blockIdx.x;

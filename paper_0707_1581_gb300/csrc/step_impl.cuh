@@ -21,25 +21,24 @@ cudaError_t step_one(const BoxStep<S> &b, const Launch &L, const uint32_t *step_
             if (L.by == 1 && (uint64_t)Q * (uint64_t)b.plane < (1ull << 32)) {
                 if constexpr (Storage<S>::stochastic) {
                     if (L.bx <= 128) {   // the register-capped kernel takes at most 128 threads a block
-                        k_stream_collide_row4<S, LAYOUT, NOISE, FORCE, V><<<grid, block, 0, st>>>(b, step_ptr, step);
-                        return cudaGetLastError();
+                        return launch_chained(k_stream_collide_row4<S, LAYOUT, NOISE, FORCE, V>, grid, block, st, b,
+                                              step_ptr, step);
                     }
                 }
-                k_stream_collide<S, LAYOUT, NOISE, FORCE, V, true, false, true><<<grid, block, 0, st>>>(b, step_ptr, step);
-            } else {
-                k_stream_collide<S, LAYOUT, NOISE, FORCE, V, true><<<grid, block, 0, st>>>(b, step_ptr, step);
+                return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, true, false, true>, grid, block,
+                                      st, b, step_ptr, step);
             }
-            return cudaGetLastError();
+            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, true>, grid, block, st, b, step_ptr,
+                                  step);
         }
     }
     if constexpr (V > 1) {
         if (L.warprow) {
-            k_stream_collide<S, LAYOUT, NOISE, FORCE, V, false, true><<<grid, block, 0, st>>>(b, step_ptr, step);
-            return cudaGetLastError();
+            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, false, true>, grid, block, st, b,
+                                  step_ptr, step);
         }
     }
-    k_stream_collide<S, LAYOUT, NOISE, FORCE, V><<<grid, block, 0, st>>>(b, step_ptr, step);
-    return cudaGetLastError();
+    return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V>, grid, block, st, b, step_ptr, step);
 }
 
 template <class S, int LAYOUT, int NOISE, bool FORCE, int V>
@@ -47,8 +46,8 @@ cudaError_t step_batch(const BatchParams<S> &P, int total_blocks, const Launch &
                        uint32_t step, cudaStream_t st)
 {
     dim3 block(L.bx, L.by, 1);
-    k_stream_collide_batch<S, LAYOUT, NOISE, FORCE, V><<<total_blocks, block, 0, st>>>(P, step_ptr, step);
-    return cudaGetLastError();
+    return launch_chained(k_stream_collide_batch<S, LAYOUT, NOISE, FORCE, V>, dim3(total_blocks), block, st, P,
+                          step_ptr, step);
 }
 
 template <class S, int LAYOUT, int NOISE, bool FORCE>
