@@ -331,9 +331,9 @@ BoxStep<S> make_step(const flb_ctx *c, const Box &b, int orient)
     s.nzl = b.cfg.nz;
     s.plane = b.plane;
     s.replica = b.cfg.replica;
-    const int sx = c->L.bx * c->L.V;
-    s.gx = (b.cfg.nx + sx - 1) / sx;
-    s.gy = (b.cfg.ny + c->L.by - 1) / c->L.by;
+    s.groups = b.cfg.nx / (c->L.V == 4 && sizeof(S) * 4 > 16 ? 2 : c->L.V);
+    s.by_groups = FastDiv(s.groups);
+    s.by_ny = FastDiv(b.cfg.ny);
     if constexpr (sizeof(typename Storage<S>::R) == 8) s.K = b.Kd;
     else s.K = b.Kf;
 #ifdef FLB_BOUNDS_CHECK
@@ -402,14 +402,13 @@ int upload_batch_tables(flb_ctx *c)
                 blocks = 0;
             }
             BoxStep<S> s = make_step<S>(c, b, o);
-            // densely packed threads: gx = x-groups per row, ceil(groups / T) blocks
-            const int V = c->L.V == 4 && sizeof(S) * 4 > 16 ? 2 : c->L.V;
-            const int T = c->L.bx * c->L.by;
-            s.gx = b.cfg.nx / V;
-            s.gy = b.cfg.ny;
-            s.warprow = V > 1 && s.gx <= 32 && 32 % s.gx == 0;
+            const int T = c->L.bx * c->L.by, g = s.groups;
+            s.warprow = c->L.V > 1 && g <= 32 && 32 % g == 0;
+            // FP32: whole rows per block; else threads packed densely over the box
+            if (c->L.V > 1 && sizeof(S) == 4 && !s.warprow && g <= T) s.rows = std::min(T / g, kXchRows);
+            const int64_t rows = (int64_t)b.cfg.ny * b.cfg.nz;
             s.block0 = blocks;
-            blocks += (int)(((int64_t)s.gx * b.cfg.ny * b.cfg.nz + T - 1) / T);
+            blocks += (int)(s.rows ? (rows + s.rows - 1) / s.rows : (rows * g + T - 1) / T);
             P->boxes[P->nboxes++] = s;
             c->batch[o].back().blocks = blocks;
         }
@@ -709,24 +708,51 @@ int usable_V(const flb_ctx *c, int V, int bx, int by)
     }
 }
 
-// The row-exchange variant: one box, 4 sites per thread, 32-bit or smaller
-// storage, each block row exactly one box row of whole warps, at most
-// kXchWarps warps per row and kXchRows rows per block.
-bool fullrow_ok(const flb_ctx *c, const Launch &L)
+// Which exchange the single-box kernel uses for a launch shape (measured, see
+// Exchange in kernels.cuh): rows that tile the warps; as many whole rows as the
+// block's threads hold -- FP32 always, the formats bound by instructions (16-bit,
+// FP64) where hardly a lane idles --; blocks that lie in one row where they cover
+// it with few idle lanes; else threads over the whole box.
+void set_exchange(const flb_ctx *c, Launch &L)
 {
-    if (c->boxes.size() != 1 || L.V != 4 || c->store == FLB_STORE_F64 || is_d2(c)) return false;
-    const int nx = c->boxes[0].cfg.nx;
-    return L.bx * L.V == nx && L.bx % 32 == 0 && L.bx / 32 <= kXchWarps && L.by <= kXchRows;
+    L.warprow = L.edgerow = false;
+    L.rows = 0;
+    if (c->boxes.size() != 1 || L.V < 2 || is_d2(c)) return;
+    const int V = (c->store == FLB_STORE_F64 && L.V == 4) ? 2 : L.V;
+    const int nx = c->boxes[0].cfg.nx, T = L.bx * L.by;
+    const int g = nx / V;
+    if (L.bx == g && 32 % g == 0 && T % 32 == 0) {
+        L.warprow = true;
+        return;
+    }
+    if (T >= g) {
+        const int rows = std::min(T / g, kXchRows);
+        const double busy = (double)rows * g / ((rows * g + 31) / 32 * 32);
+        if (c->store == FLB_STORE_F32 || busy >= (V == 4 ? 1.0 : 0.95)) {
+            L.rows = rows;
+            return;
+        }
+    }
+    L.edgerow = L.by == 1 && g >= 0.95 * ((g + T - 1) / T * T);
 }
 
-// The in-warp variant: one box, V > 1, each block row is one box row of
-// bx lanes with bx dividing 32 (and whole warps), so rows tile the warps.
-bool warprow_ok(const flb_ctx *c, const Launch &L)
+// The block of whole rows of g threads (g <= 256) that keeps most threads busy:
+// the share of its threads that own sites, times the warps an SM holds of it (at
+// 128 registers a thread, 512 threads) over 16.  96 wide (g = 24): 96 threads,
+// 35.0 GLUPS (FP32, AB) against 29.8 with 128 threads of 32 per row.
+int row_block(int g)
 {
-    if (c->boxes.size() != 1 || L.V < 2 || is_d2(c)) return false;
-    const int V = (c->store == FLB_STORE_F64 && L.V == 4) ? 2 : L.V;
-    const int nx = c->boxes[0].cfg.nx;
-    return L.bx * V == nx && 32 % L.bx == 0 && (L.bx * L.by) % 32 == 0;
+    int best = (g + 31) / 32 * 32;
+    double top = 0.0;
+    for (int rows = 1; rows <= kXchRows && rows * g <= 256; ++rows) {
+        const int T = (rows * g + 31) / 32 * 32;
+        const double busy = (double)rows * g / T * (512 / T * T / 512.0);
+        if (busy > top + 1e-9) {
+            top = busy;
+            best = T;
+        }
+    }
+    return best;
 }
 
 void default_launch(flb_ctx *c)
@@ -744,7 +770,6 @@ void default_launch(flb_ctx *c)
         const int want = f.sites_per_thread ? f.sites_per_thread : (c->store == FLB_STORE_F64 ? 2 : 4);
         L.V = usable_V(c, want, L.bx, L.by);
         if (L.V == 2 && c->store != FLB_STORE_F64) L.V = 1;   // the D2Q9 vector kernel has V = 4 (FP64: 2)
-        L.fullrow = false;
         c->L = L;
         return;
     }
@@ -756,17 +781,41 @@ void default_launch(flb_ctx *c)
         for (const Box &b : c->boxes) total += b.N;
         while (want > 1 && total / want < 100000) want /= 2;
     }
+    if (c->store == FLB_STORE_F64) want = std::min(want, 2);
     const int sites = (maxnx + want - 1) / want;
-    int bx = 32;
+    int bx = 32, by = 0;
     while (bx < sites && bx < 128) bx *= 2;
-    // short rows in one box: a row of nx / V lanes, several rows per warp
-    const int g = maxnx / want;
-    if (c->boxes.size() == 1 && maxnx % want == 0 && g < 32 && 32 % g == 0) bx = g;
+    if (c->boxes.size() == 1) {
+        const Box &b = c->boxes[0];
+        int V = want;
+        while (maxnx % V != 0) V /= 2;
+        const int g = maxnx / V;
+        if (V > 1 && g <= 32 && 32 % g == 0) {
+            bx = g;          // several rows per warp
+        } else if (!f.block_x && !f.block_y) {
+            by = 1;
+            if (V > 1) {
+                Launch r;
+                r.V = V;
+                r.by = 1;
+                r.bx = g <= 256 ? row_block(g) : 128;
+                set_exchange(c, r);
+                // blocks of one row each, of 64 to 160 threads
+                for (int nb = (g + 159) / 160; !r.rows && (nb == (g + 159) / 160 || !r.edgerow) && (g + nb - 1) / nb >= 64; ++nb) {
+                    r.bx = ((g + nb - 1) / nb + 31) / 32 * 32;
+                    set_exchange(c, r);
+                }
+                bx = r.rows || r.edgerow ? r.bx : 128;
+            }
+            // FP64 occupies the SM's FP64 unit 64 cycles per warp instruction: one-warp blocks spread a small
+            // box over the SMs (16^3: 7.8 us per step, 9.1 with 128 threads; 32^3: 14.0, 16.1)
+            else bx = c->store == FLB_STORE_F64 && b.N < 100000 ? 32 : 128;
+        }
+    }
     L.bx = f.block_x ? f.block_x : bx;
-    L.by = f.block_y ? f.block_y : std::max(1, 128 / L.bx);
+    L.by = f.block_y ? f.block_y : (by ? by : std::max(1, 128 / L.bx));
     L.V = usable_V(c, want, L.bx, L.by);
-    L.warprow = warprow_ok(c, L);
-    L.fullrow = !L.warprow && fullrow_ok(c, L);
+    set_exchange(c, L);
     c->L = L;
 }
 
@@ -1638,8 +1687,7 @@ int tune_shapes(flb_ctx *c, int trials, float *best_out)
             if (usable_V(c, L.V, L.bx, L.by) != L.V) continue;
             // the D2Q9 vector kernel has one width per format
             if (is_d2(c) && L.V != 1 && L.V != (c->store == FLB_STORE_F64 ? 2 : 4)) continue;
-            L.warprow = warprow_ok(c, L);
-            L.fullrow = !L.warprow && fullrow_ok(c, L);
+            set_exchange(c, L);
             if (L.bx * L.V > 2 * std::max(32, maxnx)) continue;   // mostly idle threads
             c->L = L;
             if ((rc = refresh_batch_tables(c)) != FLB_OK) break;
@@ -1766,8 +1814,7 @@ int flb_set_launch(flb_ctx *c, int V, int bx, int by)
     L.V = V;
     L.bx = bx;
     L.by = by;
-    L.warprow = warprow_ok(c, L);
-    L.fullrow = !L.warprow && fullrow_ok(c, L);
+    set_exchange(c, L);
     c->L = L;
     drop_graphs(c);
     return refresh_batch_tables(c);

@@ -568,18 +568,13 @@ struct Storage<bf16sr> {
     __device__ static double to_double(bf16sr v) { return (double)load(v); }
 };
 
-// Load of one stored element (the 16-bit pattern for bf16sr).  An ordinary
-// load: a step's kernel starts while the one before it still writes (see
-// wait_for_previous_step), which the read-only path does not allow.
+// Load of one stored element.  An ordinary load: a step's kernel starts while
+// the one before it still writes (see wait_for_previous_step), which the
+// read-only path does not allow.
 template <class S>
 __device__ __forceinline__ S load_ro(const S *p)
 {
     return *p;
-}
-template <>
-__device__ __forceinline__ bf16sr load_ro<bf16sr>(const bf16sr *p)
-{
-    return bf16sr{*reinterpret_cast<const unsigned short *>(p)};
 }
 
 // Stochastic rounding of x to bfloat16 with 16 random bits r: r is added to

@@ -29,8 +29,10 @@ struct Launch {
     int V = 1;        // x-consecutive sites per thread
     int bx = 64;      // block threads along x
     int by = 4;       // block threads along y
-    bool fullrow = false;   // one box, bx * V == nx, whole warps: edge exchange inside the block
-    bool warprow = false;   // one box, bx * V == nx, bx divides 32: rows tile the warps, shuffles only
+    // one box, V > 1 (neither: bx * by threads over the box, scalar accesses at row and warp ends):
+    bool warprow = false;   // bx * V == nx, bx divides 32: rows tile the warps, shuffles only
+    int rows = 0;           // > 0: whole rows of nx / V threads per block (at most kXchRows)
+    bool edgerow = false;   // blocks of one row each, scalar accesses at row and warp ends
 };
 
 // Launches a step kernel with programmatic stream serialization: its blocks may

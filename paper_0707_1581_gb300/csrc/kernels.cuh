@@ -19,17 +19,35 @@ namespace flb {
 // In the AA steps every thread writes exactly the locations it read, so the
 // in-place update has no races whatever the launch shape.
 // --------------------------------------------------------------------------
+// n / d for 0 <= n < 2^31 and d >= 1 without a division: with 2^s >= d > 2^(s -
+// 1) and m = floor(2^(31 + s) / d) + 1 (which fits 32 bits), m d exceeds 2^(31 +
+// s) by at most d <= 2^s, so floor(n m / 2^(31 + s)) is the quotient.
+struct FastDiv {
+    uint32_t mul;
+    int shift;
+    FastDiv() = default;
+    __host__ explicit FastDiv(int d)
+    {
+        int s = 0;
+        while ((1ll << s) < d) ++s;
+        shift = 31 + s;
+        mul = (uint32_t)((1ull << shift) / (uint64_t)d + 1);
+    }
+    __device__ __forceinline__ int quot(int n) const { return (int)(((uint64_t)(uint32_t)n * mul) >> shift); }
+};
+
 template <class S>
 struct BoxStep {
     const S *src;
     S *dst;
     int nx, ny, nz;
-    int warprow;               // batched launch: nx / V divides 32, rows tile the warps (see update_vec)
+    int warprow;               // batched launch: nx / V divides 32, rows tile the warps (kWarpRow)
     int64_t plane;             // elements between population planes
     uint32_t replica;
-    int gx, gy;                // blocks along x and y of this box (batched launch)
     int block0;                // first block of this box in a batched launch
     int z0, nzl;               // single-box launch: planes z0 .. z0 + nzl - 1 (grid.z = nzl)
+    int groups, rows;          // threads (of V sites) per row; whole rows per block (kRows)
+    FastDiv by_groups, by_ny;  // division by groups and by ny
     CollideConsts<typename Storage<S>::R> K;
     FLB_VIOL_FIELD
 };
@@ -244,37 +262,86 @@ __device__ __forceinline__ R shfl_down1(R v)
     return __shfl_down_sync(0xffffffffu, v, 1);
 }
 
-// Row-edge exchange of a block whose rows are covered by whole warps: slot
-// [ty][i][w] of warp w in block row ty, for the load phase (l*) and the store
-// phase (s*).  At most kXchRows block rows and kXchWarps warps per row.
-constexpr int kXchRows = 2, kXchWarps = 8;
-template <class R>
+// How update_vec gets the elements that cross from one thread's V sites into
+// the next's (the x-shift by c_x = +-1).
+//   kEdges    lane - 1 and lane + 1 by shuffle where they own the adjacent
+//             sites, else by scalar accesses; any shape.
+//   kEdgeRow  the same, in blocks that lie in one row.
+//   kOneRow   the block is one box row of whole warps: shuffles inside a warp,
+//             a shared-memory exchange across warps and around the periodic row
+//             end; every lane reads and writes only whole aligned vectors.
+//   kRagRow   the block is one box row that is not whole warps: as kOneRow, with
+//             an exchange slot for the row end besides the one per warp end.
+//   kRows     the block is several whole box rows: as kRagRow, a slot per row.
+//   kWarpRow  a row is g = nx / V consecutive lanes and g divides 32, so rows
+//             tile the warps: every neighbour element comes by an indexed
+//             shuffle, with no edge access and no shared memory.
+// FP32, bound by memory, gains most from the whole vectors: 250 x 187 x 93 AA
+// 117 us per step with kEdges, 100 with kRagRow; 300 x 200 x 60 AB 96 / 84 (kRows);
+// 640 x 320 x 40 AB 207 / 181 (kOneRow).  The 16-bit formats, bound by
+// instructions, only where no lane idles: 300 x 200 x 60 AB 61.7 / 66.3, 400 x
+// 100 x 100 64.5 / 76.1 (kRagRow, 100 of 128 lanes), 640 wide 132 / 129; two sites
+// per thread 87 / 77 (250 wide AA).  FP64 likewise: 90 x 100 x 110 368 / 397 (90 of
+// 96 lanes), 72^3 154 / 145.  (set_exchange in api.cu decides.)
+enum Exchange : int { kEdges = 0, kOneRow = 1, kRows = 2, kWarpRow = 3, kRagRow = 4, kEdgeRow = 5 };
+
+// The block's exchange memory: what a warp (kOneRow) or a warp or row (kRows)
+// hands over its ends, in the load phase (l*, as stored) and in the store phase
+// (s*).
+constexpr int kXchWarps = 8;       // warps per block, at most
+constexpr int kXchRows = 32;       // rows per block, at most
+template <class S, int XCH>
 struct RowExchange {
-    R l_last[kXchRows][Q][kXchWarps];    // last element of each warp's vector (pull from x - 1)
-    R l_first[kXchRows][Q][kXchWarps];   // first element (pull from x + 1)
-    R s_last[kXchRows][Q][kXchWarps];    // value pushed to x + 1 across the warp edge
-    R s_first[kXchRows][Q][kXchWarps];   // value pushed to x - 1 across the warp edge
+    using R = typename Storage<S>::R;
+    static constexpr int kRowSlots = XCH == kRows ? kXchRows : 1;
+    static constexpr int kSlots = XCH == kOneRow ? kXchWarps : kRowSlots + kXchWarps;
+    S l_last[Q][kSlots];    // last element of the vector (pull from x - 1)
+    S l_first[Q][kSlots];   // first element (pull from x + 1)
+    R s_last[Q][kSlots];    // value pushed to x + 1 across the end
+    R s_first[Q][kSlots];   // value pushed to x - 1 across the end
 };
 
-// FULLROW: every block row is exactly one box row (blockDim.x * V == nx, whole
-// warps), so the neighbour of every edge element is in the block: shuffles
-// inside a warp, the exchange above across warps (and around the periodic
-// row end), and every lane reads and writes only whole aligned vectors.
-// WARPROW: the converse -- a row is g = nx / V consecutive lanes and g divides
-// 32, so rows tile the warps and the periodic neighbour of a row end is in the
-// same warp: every neighbour element comes by an indexed shuffle (lane - 1,
-// or lane + g - 1 at the row start; lane + 1, or lane - g + 1 at the row end),
-// with no edge access and no shared memory.
+// A thread's place in its block's rows (kOneRow, kRows): which ends it owns,
+// and the exchange slots that it writes (mine_*) and reads (from_*).  A row end
+// has the row's slot; a warp end inside a row has the warp's.
+struct RowPlace {
+    bool give_last, give_first;    // the right (left) neighbour cannot reach this thread by shuffle
+    bool take_left, take_right;    // the left (right) neighbour's element comes from the exchange
+    int mine_last, mine_first, from_left, from_right;
+};
+template <int XCH>
+__device__ __forceinline__ RowPlace row_place(int lane, int warp, int nwarp, int tx, int g, int row)
+{
+    RowPlace p;
+    if constexpr (XCH == kOneRow) {
+        p.give_last = p.take_right = lane == 31;
+        p.give_first = p.take_left = lane == 0;
+        p.mine_last = p.mine_first = warp;
+        p.from_left = warp == 0 ? nwarp - 1 : warp - 1;
+        p.from_right = warp == nwarp - 1 ? 0 : warp + 1;
+    } else {
+        constexpr int kRowSlots = XCH == kRows ? kXchRows : 1;
+        const bool start = tx == 0, end = tx == g - 1;
+        p.give_last = p.take_right = lane == 31 || end;
+        p.give_first = p.take_left = lane == 0 || start;
+        p.mine_last = end ? row : kRowSlots + warp;
+        p.mine_first = start ? row : kRowSlots + warp;
+        p.from_left = start ? row : kRowSlots + (lane == 0 ? warp - 1 : warp);
+        p.from_right = end ? row : kRowSlots + (lane == 31 ? warp + 1 : warp);
+    }
+    return p;
+}
+
 // OFF32: every element offset of the box's buffer (Q planes) fits in 32 bits,
 // so an address is one 32-bit offset (slot, row and x together) added to the
 // buffer pointer, instead of 64-bit arithmetic per access.
-template <class S, int LAYOUT, int NOISE, bool FORCE, int V, bool FULLROW = false, bool WARPROW = false,
-          bool OFF32 = false>
+// row: the thread's row within its block (kRows).
+template <class S, int LAYOUT, int NOISE, bool FORCE, int V, int XCH = kEdges, bool OFF32 = false>
 __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, int z, bool active, bool left_in_warp,
-                                           bool right_in_warp, uint32_t step,
-                                           RowExchange<typename Storage<S>::R> *xch = nullptr)
+                                           bool right_in_warp, uint32_t step, RowExchange<S, XCH> *xch = nullptr,
+                                           int row = 0)
 {
-    static_assert(!(FULLROW && WARPROW), "one row-exchange variant at a time");
+    constexpr bool FULLROW = XCH == kOneRow || XCH == kRows || XCH == kRagRow, WARPROW = XCH == kWarpRow;
     using R = typename Storage<S>::R;
     // element (slot, row offset + x) of the source / destination buffer
     auto src_at = [&](int slot, int off) -> const S * {
@@ -290,17 +357,6 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
     const int yo[3] = {(y == 0 ? ny - 1 : y - 1) * nx, y * nx, (y == ny - 1 ? 0 : y + 1) * nx};
     const int nxy = nx * ny;
     const int zo[3] = {(z == 0 ? nz - 1 : z - 1) * nxy, z * nxy, (z == nz - 1 ? 0 : z + 1) * nxy};
-    // a neighbour's element comes by shuffle only inside the same row
-    const bool shl = left_in_warp && x0 != 0;          // lane - 1 owns x0 - V .. x0 - 1
-    const bool shr = right_in_warp && x0 + V != nx;    // lane + 1 owns x0 + V .. x0 + 2V - 1
-    const int x_left = x0 == 0 ? nx - 1 : x0 - 1;      // element left of the group (periodic)
-    const int x_right = x0 + V == nx ? 0 : x0 + V;     // element right of the group (periodic)
-    // every lane reads its edge element with the vector (no wait behind the
-    // shuffle, no divergence); lanes that get it by shuffle re-read a word of
-    // their own vector instead
-    const int x_lload = shl ? x0 : x_left;
-    const int x_rload = shr ? x0 + V - 1 : x_right;
-
     const uint32_t site0 = (uint32_t)(zo[1] + yo[1]) + (uint32_t)x0;
     // Two sites per thread in rows of whole warps (the small boxes): the normals,
     // which need no stored state, before the wait; four sites' would not fit
@@ -318,6 +374,17 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
         for (int v = 0; v < V; ++v) draw_normals<R>(B.K, site0 + v, step, B.replica, g[v]);
     }
     wait_for_previous_step();
+
+    // a neighbour's element comes by shuffle only inside the same row
+    const bool shl = left_in_warp && x0 != 0;          // lane - 1 owns x0 - V .. x0 - 1
+    const bool shr = right_in_warp && x0 + V != nx;    // lane + 1 owns x0 + V .. x0 + 2V - 1
+    const int x_left = x0 == 0 ? nx - 1 : x0 - 1;      // element left of the group (periodic)
+    const int x_right = x0 + V == nx ? 0 : x0 + V;     // element right of the group (periodic)
+    // every lane reads its edge element with the vector (no wait behind the
+    // shuffle, no divergence); lanes that get it by shuffle re-read a word of
+    // their own vector instead
+    const int x_lload = shl ? x0 : x_left;
+    const int x_rload = shr ? x0 + V - 1 : x_right;
 
     // 1. issue every load of the 19 planes (vector + edge element) before
     //    any shuffle, so that all of them are in flight together
@@ -338,29 +405,30 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
         if (!FULLROW && !WARPROW && LAYOUT != kAAEven && cx > 0) edge[i] = load_ro(FLB_GUARD_LD(B, src_at(slot, ro + x_lload), 1));
         if (!FULLROW && !WARPROW && LAYOUT != kAAEven && cx < 0) edge[i] = load_ro(FLB_GUARD_LD(B, src_at(slot, ro + x_rload), 1));
     }
-    const int lane = (threadIdx.y * blockDim.x + threadIdx.x) & 31;
+    const int lane = (threadIdx.y * blockDim.x + threadIdx.x) & 31;   // 2-D blocks: kWarpRow only
     // WARPROW source lanes of the left (x - 1) and right (x + 1) neighbour, periodic in the row
     const int gl = nx / V;
     const int lane_l = WARPROW ? (x0 != 0 ? lane - 1 : lane + gl - 1) : 0;
     const int lane_r = WARPROW ? (x0 + V != nx ? lane + 1 : lane - gl + 1) : 0;
-    const int warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5, row_t = threadIdx.y;
-    if (FULLROW && LAYOUT != kAAEven) {
-        // publish each warp's edge elements, then read the neighbours' (periodic in the row)
+    const RowPlace at = FULLROW ? row_place<XCH>(lane, (int)threadIdx.x >> 5, (int)blockDim.x >> 5, x0 / V, gl, row)
+                                : RowPlace{};
+    if constexpr (FULLROW && LAYOUT != kAAEven) {
+        // publish the end elements, then read the neighbours' (periodic in the row)
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            if (vel_x(i) > 0 && lane == 31) xch->l_last[row_t][i][warp] = Storage<S>::load(raw[i][V - 1]);
-            if (vel_x(i) < 0 && lane == 0) xch->l_first[row_t][i][warp] = Storage<S>::load(raw[i][0]);
+            if (vel_x(i) > 0 && at.give_last && (XCH == kOneRow || active)) xch->l_last[i][at.mine_last] = raw[i][V - 1];
+            if (vel_x(i) < 0 && at.give_first && (XCH == kOneRow || active)) xch->l_first[i][at.mine_first] = raw[i][0];
         }
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            if (vel_x(i) > 0) edge[i] = Storage<S>::store(xch->l_last[row_t][i][warp == 0 ? nwarp - 1 : warp - 1]);
-            if (vel_x(i) < 0) edge[i] = Storage<S>::store(xch->l_first[row_t][i][warp == nwarp - 1 ? 0 : warp + 1]);
+            if (vel_x(i) > 0) edge[i] = xch->l_last[i][at.from_left];
+            if (vel_x(i) < 0) edge[i] = xch->l_first[i][at.from_right];
         }
     }
     // 2. shift the planes with c_x != 0 by one site
-    const bool use_left = FULLROW ? lane != 0 : shl;
-    const bool use_right = FULLROW ? lane != 31 : shr;
+    const bool use_left = FULLROW ? !at.take_left : shl;
+    const bool use_right = FULLROW ? !at.take_right : shr;
     R f[V][Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -418,19 +486,19 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
     for (int v = 0; v < V; ++v) stochastic_round<S>(f[v], site0 + v, step, B.replica, B.K.rk0, B.K.rk1);
 
     if constexpr (kStart<S, V> == kBeforeStores) let_next_step_start();
-    R pushed[Q];   // FULLROW, AA odd: the value crossing into this warp's vector from the neighbour warp
-    if (FULLROW && LAYOUT == kAAOdd) {
+    R pushed[Q];   // FULLROW, AA odd: the value that crosses into this thread's vector through the exchange
+    if constexpr (FULLROW && LAYOUT == kAAOdd) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            if (vel_x(i) > 0 && lane == 31) xch->s_last[row_t][i][warp] = f[V - 1][i];
-            if (vel_x(i) < 0 && lane == 0) xch->s_first[row_t][i][warp] = f[0][i];
+            if (vel_x(i) > 0 && at.give_last && (XCH == kOneRow || active)) xch->s_last[i][at.mine_last] = f[V - 1][i];
+            if (vel_x(i) < 0 && at.give_first && (XCH == kOneRow || active)) xch->s_first[i][at.mine_first] = f[0][i];
         }
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             pushed[i] = R(0);
-            if (vel_x(i) > 0) pushed[i] = xch->s_last[row_t][i][warp == 0 ? nwarp - 1 : warp - 1];
-            if (vel_x(i) < 0) pushed[i] = xch->s_first[row_t][i][warp == nwarp - 1 ? 0 : warp + 1];
+            if (vel_x(i) > 0) pushed[i] = xch->s_last[i][at.from_left];
+            if (vel_x(i) < 0) pushed[i] = xch->s_first[i][at.from_right];
         }
     }
 #pragma unroll
@@ -457,14 +525,14 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
             S out[V];
             if (cx > 0) {   // site x goes to x + 1
                 const R from_left = shfl_up1(f[V - 1][i]);
-                out[0] = Storage<S>::store(lane == 0 ? pushed[i] : from_left);
+                out[0] = Storage<S>::store(at.take_left ? pushed[i] : from_left);
 #pragma unroll
                 for (int v = 1; v < V; ++v) out[v] = Storage<S>::store(f[v - 1][i]);
             } else {        // site x goes to x - 1
                 const R from_right = shfl_down1(f[0][i]);
 #pragma unroll
                 for (int v = 0; v < V - 1; ++v) out[v] = Storage<S>::store(f[v + 1][i]);
-                out[V - 1] = Storage<S>::store(lane == 31 ? pushed[i] : from_right);
+                out[V - 1] = Storage<S>::store(at.take_right ? pushed[i] : from_right);
             }
             S *p = dst_at(i, zo[1 + cz] + yo[1 + cy] + x0);
             store_vec_when<S, V>(active && FLB_GUARD_ST(B, p, V), p, out);
@@ -511,86 +579,102 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
     }
 }
 
-// Lane bookkeeping of a (bx, by) block for update_vec: the thread left
-// (right) of (tx, ty) in the row is lane - 1 (+ 1) of the same warp unless tx
-// or the lane sits on an edge.
-struct LaneEdges {
-    bool left, right;
-};
-__device__ __forceinline__ LaneEdges lane_edges()
-{
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int lane = tid & 31;
-    return LaneEdges{threadIdx.x > 0 && lane > 0, threadIdx.x + 1 < blockDim.x && lane < 31};
-}
-
 __device__ __forceinline__ uint32_t step_of(const uint32_t *step_ptr, uint32_t step)
 {
     return step_ptr ? __ldg(step_ptr) + step : step;
 }
 
-// One box: grid (gx, gy, nz), block (bx, by); thread (tx, ty) updates the V
-// sites x0 = V (blockIdx.x bx + tx) .. x0 + V - 1 of row (y, z).  V = 1 is the
-// general scalar path; V > 1 needs nx % V == 0.  UROW (FULLROW with by = 1
-// and a buffer of fewer than 2^32 elements): the block is one whole box row,
-// y = blockIdx.y, so the row offsets of the nine neighbour rows are the same
-// for the whole block, and every address is one 32-bit element offset.
-template <class S, int LAYOUT, int NOISE, bool FORCE, int V, bool FULLROW, bool WARPROW, bool UROW>
+// Block b of a kRows launch: rows b B.rows .. of the box's planes z0 .. z0 + nzl - 1,
+// thread tid on group tid mod B.groups of row tid / B.groups.
+template <class S, int LAYOUT, int NOISE, bool FORCE, int V, bool OFF32>
+__device__ __forceinline__ void update_rows(const BoxStep<S> &B, int tid, int b, uint32_t step,
+                                            RowExchange<S, kRows> &xch)
+{
+    const int tr = B.by_groups.quot(tid), tx = tid - tr * B.groups;
+    const int first = b * B.rows, nrows = B.ny * B.nzl;
+    const bool active = tr < B.rows && first + tr < nrows;
+    const int row = active ? first + tr : min(first, nrows - 1);   // in bounds for every lane
+    const int zr = B.by_ny.quot(row);
+    update_vec<S, LAYOUT, NOISE, FORCE, V, kRows, OFF32>(B, V * tx, row - zr * B.ny, B.z0 + zr, active, true, true, step,
+                                                         &xch, min(tr, kXchRows - 1));
+}
+
+// One box; a thread updates the V sites x0 .. x0 + V - 1 of row (y, z); V > 1
+// needs nx % V == 0 and blocks of whole warps.
+//   kEdges   (and V = 1) a 1-D grid over the groups of V sites of all the rows
+//            of the launch, so that no lane idles at a row end.
+//   kRows    a 1-D grid over the rows of the launch (y + ny z), B.rows whole
+//            rows of B.groups threads per block; the threads beyond them (less
+//            than a warp, or rows past the last) only keep the warps whole.
+//   the rest grid (x, y, z), block (bx, by); kOneRow, kRagRow, kEdgeRow: y =
+//            blockIdx.y, so the row offsets of the nine neighbour rows are the
+//            same for the whole block (1000 x 100 x 40 FP16 AB: 65.6 us per step
+//            with kEdgeRow, 71.6 with kEdges).
+template <class S, int LAYOUT, int NOISE, bool FORCE, int V, int XCH, bool OFF32>
 __device__ __forceinline__ void stream_collide_box(const BoxStep<S> &B, const uint32_t *step_ptr, uint32_t step)
 {
-    static_assert(!UROW || FULLROW, "UROW is a FULLROW launch");
     if constexpr (kStart<S, V> == kAtStart) let_next_step_start();
-    int x0 = V * (blockIdx.x * blockDim.x + threadIdx.x);
-    int y = UROW ? (int)blockIdx.y : (int)(blockIdx.y * blockDim.y + threadIdx.y);
-    const int z = B.z0 + (int)blockIdx.z;
-    if constexpr (V == 1) {
-        if (x0 >= B.nx || y >= B.ny) return;
-        update_sites<S, LAYOUT, NOISE, FORCE, 1>(B, x0, y, z, step_of(step_ptr, step));
-    } else {
-        const bool active = x0 < B.nx && y < B.ny;
-        if (!active) {   // stay in the warp for the shuffles, on an in-bounds position
-            x0 = min(x0, B.nx - V);
-            y = min(y, B.ny - 1);
-        }
-        const LaneEdges e = lane_edges();
-        if constexpr (FULLROW) {
-            __shared__ RowExchange<typename Storage<S>::R> xch;
-            update_vec<S, LAYOUT, NOISE, FORCE, V, true, false, UROW>(B, x0, y, z, active, e.left, e.right,
-                                                                      step_of(step_ptr, step), &xch);
-        } else if constexpr (WARPROW) {
-            update_vec<S, LAYOUT, NOISE, FORCE, V, false, true>(B, x0, y, z, active, e.left, e.right,
-                                                                step_of(step_ptr, step));
+    const int tid = (int)threadIdx.x, lane = tid & 31;
+    if constexpr (XCH == kRows) {
+        __shared__ RowExchange<S, XCH> xch;
+        update_rows<S, LAYOUT, NOISE, FORCE, V, OFF32>(B, tid, (int)blockIdx.x, step_of(step_ptr, step), xch);
+    } else if constexpr (XCH == kEdges) {
+        const uint32_t items = (uint32_t)B.groups * (uint32_t)(B.ny * B.nzl);
+        const uint32_t it = blockIdx.x * blockDim.x + threadIdx.x;
+        const bool active = it < items;
+        const int item = (int)(active ? it : items - 1);   // idle lanes work on the last group, store nothing
+        const int row = B.by_groups.quot(item), xg = item - row * B.groups;
+        const int zr = B.by_ny.quot(row);
+        if constexpr (V == 1) {
+            if (active)
+                update_sites<S, LAYOUT, NOISE, FORCE, 1>(B, xg, row - zr * B.ny, B.z0 + zr, step_of(step_ptr, step));
         } else {
-            update_vec<S, LAYOUT, NOISE, FORCE, V>(B, x0, y, z, active, e.left, e.right, step_of(step_ptr, step));
+            // consecutive lanes own consecutive groups: lane - 1 holds x0 - V whenever x0 > 0
+            update_vec<S, LAYOUT, NOISE, FORCE, V, XCH, OFF32>(B, V * xg, row - zr * B.ny, B.z0 + zr, active, lane > 0,
+                                                               lane < 31, step_of(step_ptr, step));
         }
+    } else if constexpr (XCH == kWarpRow) {
+        const int y = (int)(blockIdx.y * blockDim.y + threadIdx.y);
+        update_vec<S, LAYOUT, NOISE, FORCE, V, XCH, OFF32>(B, V * tid, min(y, B.ny - 1), B.z0 + (int)blockIdx.z, y < B.ny,
+                                                           true, true, step_of(step_ptr, step));
+    } else if constexpr (XCH == kEdgeRow) {
+        const int x0 = V * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+        update_vec<S, LAYOUT, NOISE, FORCE, V, XCH, OFF32>(B, min(x0, B.nx - V), (int)blockIdx.y, B.z0 + (int)blockIdx.z,
+                                                           x0 < B.nx, lane > 0, lane < 31, step_of(step_ptr, step));
+    } else {
+        __shared__ RowExchange<S, XCH> xch;
+        const bool active = XCH == kOneRow || tid < B.groups;
+        update_vec<S, LAYOUT, NOISE, FORCE, V, XCH, OFF32>(B, V * (XCH == kOneRow ? tid : min(tid, B.groups - 1)),
+                                                           (int)blockIdx.y, B.z0 + (int)blockIdx.z, active, true, true,
+                                                           step_of(step_ptr, step), &xch);
     }
 }
 
-template <class S, int LAYOUT, int NOISE, bool FORCE, int V, bool FULLROW = false, bool WARPROW = false,
-          bool UROW = false>
-__global__ void __launch_bounds__(256) k_stream_collide(const BoxStep<S> B, const uint32_t *step_ptr, uint32_t step)
+// Registers: 512 threads per SM (at most 128 each) with four sites per thread --
+// left free, many variants took 130 to 176, which leaves room for three or two
+// blocks of 128 threads instead of four (the stochastically rounded AA odd step
+// took 130 and ran 15 % slower) -- and 768 (at most 85) with two, which took 120
+// (250 x 187 x 93 AA, per step: FP16 90.6 -> 77.3 us, FP32 107 -> 100; 64
+// registers: 76.8 and 100.5).  The small boxes of kWarpRow hold their normals
+// too and keep what they take (64^3 FP32 AA 6.2 us, 6.8 with 85).
+template <class S, int V, int XCH>
+constexpr int kMinBlocks = sizeof(S) == 8 ? 1 : (V == 4 ? 2 : (V == 2 && XCH != kWarpRow ? 3 : 1));
+
+template <class S, int LAYOUT, int NOISE, bool FORCE, int V, int XCH = kEdges, bool OFF32 = false>
+__global__ void __launch_bounds__(256, kMinBlocks<S, V, XCH>) k_stream_collide(const BoxStep<S> B,
+                                                                             const uint32_t *step_ptr, uint32_t step)
 {
-    stream_collide_box<S, LAYOUT, NOISE, FORCE, V, FULLROW, WARPROW, UROW>(B, step_ptr, step);
+    stream_collide_box<S, LAYOUT, NOISE, FORCE, V, XCH, OFF32>(B, step_ptr, step);
 }
 
-// The one-row launch of the stochastically rounded format, held to four
-// 128-thread blocks per SM (at most 128 registers): left free, its AA odd step
-// took 130 registers, which left room for three blocks, and ran 15 % slower.
-template <class S, int LAYOUT, int NOISE, bool FORCE, int V>
-__global__ void __launch_bounds__(128, 4) k_stream_collide_row4(const BoxStep<S> B, const uint32_t *step_ptr,
-                                                                uint32_t step)
-{
-    stream_collide_box<S, LAYOUT, NOISE, FORCE, V, true, false, true>(B, step_ptr, step);
-}
-
-// Many boxes in one 1-D grid: box b owns blocks [block0, block0 + ceil(gx ny nz / T)),
-// T threads per block.  Inside a box the threads are packed densely: thread
-// item k = (block - block0) T + tid owns the V sites of x-group k mod gx
-// (gx = nx / V groups per row) of row k / gx, so a warp may span several
-// short rows and no lane idles at a row end; the lanes at a row start or end
-// exchange through edge loads instead of shuffles.  The box table is a kernel
-// parameter (constant bank, at most ~31 KB); batches larger than one table
-// are split into several launches.
+// Many boxes in one 1-D grid: box b owns the blocks from block0 on.  FP32 boxes
+// whose rows do not tile the warps take whole rows per block (kRows: 12 boxes of
+// 96^3, AB, 45.5 GLUPS against 39.9 with the scalar accesses of kEdges); in the
+// other boxes the threads are packed densely: thread item k = (block - block0) T
+// + tid owns the V sites of x-group k mod groups (nx / V groups per row) of row k
+// / groups, so a warp may span several short rows and no lane idles at a row
+// end.  The box table is a kernel parameter (constant bank, at most ~31 KB);
+// batches larger than one table are split into several launches.
 template <class S>
 constexpr int batch_chunk()
 {
@@ -606,8 +690,8 @@ struct BatchParams {
 };
 
 template <class S, int LAYOUT, int NOISE, bool FORCE, int V>
-__global__ void __launch_bounds__(256) k_stream_collide_batch(const __grid_constant__ BatchParams<S> P,
-                                                              const uint32_t *step_ptr, uint32_t step)
+__global__ void __launch_bounds__(256, kMinBlocks<S, V, kEdges>)
+k_stream_collide_batch(const __grid_constant__ BatchParams<S> P, const uint32_t *step_ptr, uint32_t step)
 {
     if constexpr (kStart<S, V> == kAtStart) let_next_step_start();
     // last box with block0 <= blockIdx.x (the same for the whole block)
@@ -619,14 +703,20 @@ __global__ void __launch_bounds__(256) k_stream_collide_batch(const __grid_const
         else hi = mid - 1;
     }
     const BoxStep<S> &sb = P.boxes[lo];
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int total = sb.gx * sb.ny * sb.nz;                 // x-groups of the box
-    const int item = (b - sb.block0) * (int)(blockDim.x * blockDim.y) + tid;
+    const int tid = (int)threadIdx.x;
+    if constexpr (V > 1 && sizeof(S) == 4) {
+        __shared__ RowExchange<S, kRows> xch;
+        if (sb.rows > 0) {
+            update_rows<S, LAYOUT, NOISE, FORCE, V, false>(sb, tid, b - sb.block0, step_of(step_ptr, step), xch);
+            return;
+        }
+    }
+    const int total = sb.groups * sb.ny * sb.nz;             // x-groups of the box
+    const int item = (b - sb.block0) * (int)blockDim.x + tid;
     const bool active = item < total;
     const int it = active ? item : total - 1;                // idle lanes work on the last group, store nothing
-    const int xg = it % sb.gx, row = it / sb.gx;
-    const int y = row % sb.ny, z = row / sb.ny;
-    const int x0 = V * xg;
+    const int row = sb.by_groups.quot(it), z = sb.by_ny.quot(row);
+    const int y = row - z * sb.ny, x0 = V * (it - row * sb.groups);
     if constexpr (V == 1) {
         if (!active) return;
         update_sites<S, LAYOUT, NOISE, FORCE, 1>(sb, x0, y, z, step_of(step_ptr, step));
@@ -634,7 +724,7 @@ __global__ void __launch_bounds__(256) k_stream_collide_batch(const __grid_const
         // consecutive lanes own consecutive x-groups: lane - 1 holds x0 - V whenever x0 > 0
         const int lane = tid & 31;
         if (sb.warprow)
-            update_vec<S, LAYOUT, NOISE, FORCE, V, false, true>(sb, x0, y, z, active, lane > 0, lane < 31,
+            update_vec<S, LAYOUT, NOISE, FORCE, V, kWarpRow>(sb, x0, y, z, active, lane > 0, lane < 31,
                                                                 step_of(step_ptr, step));
         else
             update_vec<S, LAYOUT, NOISE, FORCE, V>(sb, x0, y, z, active, lane > 0, lane < 31, step_of(step_ptr, step));

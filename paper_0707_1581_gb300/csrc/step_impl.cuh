@@ -13,39 +13,44 @@ namespace detail {
 template <class S, int LAYOUT, int NOISE, bool FORCE, int V>
 cudaError_t step_one(const BoxStep<S> &b, const Launch &L, const uint32_t *step_ptr, uint32_t step, cudaStream_t st)
 {
-    const int sites_x = L.bx * V;
-    dim3 grid((b.nx + sites_x - 1) / sites_x, (b.ny + L.by - 1) / L.by, b.nzl);
-    dim3 block(L.bx, L.by, 1);
-    if constexpr (V == 4 && sizeof(S) <= 4) {
-        if (L.fullrow) {
-            if (L.by == 1 && (uint64_t)Q * (uint64_t)b.plane < (1ull << 32)) {
-                if constexpr (Storage<S>::stochastic) {
-                    if (L.bx <= 128) {   // the register-capped kernel takes at most 128 threads a block
-                        return launch_chained(k_stream_collide_row4<S, LAYOUT, NOISE, FORCE, V>, grid, block, st, b,
-                                              step_ptr, step);
-                    }
-                }
-                return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, true, false, true>, grid, block,
-                                      st, b, step_ptr, step);
-            }
-            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, true>, grid, block, st, b, step_ptr,
+    const int g = b.nx / V, T = L.bx * L.by;
+    if constexpr (V > 1) {
+        const bool off32 = (uint64_t)Q * (uint64_t)b.plane < (1ull << 32);
+        if (L.warprow)
+            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, kWarpRow>,
+                                  dim3(1, (b.ny + L.by - 1) / L.by, b.nzl), dim3(L.bx, L.by), st, b, step_ptr, step);
+        if (L.rows == 1 && off32 && b.ny <= 65535) {
+            const dim3 grid(1, b.ny, b.nzl), block((g + 31) / 32 * 32);
+            if (g % 32 == 0)
+                return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, kOneRow, true>, grid, block, st, b,
+                                      step_ptr, step);
+            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, kRagRow, true>, grid, block, st, b,
+                                  step_ptr, step);
+        }
+        if (L.rows > 0) {
+            BoxStep<S> r = b;
+            r.rows = L.rows;
+            const int64_t nrows = (int64_t)b.ny * b.nzl;
+            const dim3 grid((unsigned)((nrows + L.rows - 1) / L.rows)), block((L.rows * g + 31) / 32 * 32);
+            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, kRows>, grid, block, st, r, step_ptr,
                                   step);
         }
     }
     if constexpr (V > 1) {
-        if (L.warprow) {
-            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, false, true>, grid, block, st, b,
-                                  step_ptr, step);
-        }
+        if (L.edgerow && b.ny <= 65535)
+            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, kEdgeRow>,
+                                  dim3((g + T - 1) / T, b.ny, b.nzl), dim3(T), st, b, step_ptr, step);
     }
-    return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V>, grid, block, st, b, step_ptr, step);
+    const int64_t items = (int64_t)g * b.ny * b.nzl;
+    return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V>, dim3((unsigned)((items + T - 1) / T)), dim3(T),
+                          st, b, step_ptr, step);
 }
 
 template <class S, int LAYOUT, int NOISE, bool FORCE, int V>
 cudaError_t step_batch(const BatchParams<S> &P, int total_blocks, const Launch &L, const uint32_t *step_ptr,
                        uint32_t step, cudaStream_t st)
 {
-    dim3 block(L.bx, L.by, 1);
+    const dim3 block(L.bx * L.by);
     return launch_chained(k_stream_collide_batch<S, LAYOUT, NOISE, FORCE, V>, dim3(total_blocks), block, st, P,
                           step_ptr, step);
 }

@@ -56,3 +56,64 @@ def test_chained_steps_of_a_batch_of_several_launches_per_step():
     with flb.flb_create_batch(cfgs) as ctx:
         ctx.flb_step(20)
         assert all(np.array_equal(raw(ctx, b), want[b]) for b in range(70))
+
+
+# (nx, sites per thread, block): the exchanges of the single-box kernel, with row counts that are and are not
+# multiples of the rows of a block, rows shorter than a warp, longer, and of whole warps
+SHAPES = [(12, 4, (128, 1)), (20, 4, (96, 1)), (40, 4, (128, 1)), (96, 4, (96, 1)), (100, 4, (256, 1)),
+          (132, 4, (64, 1)), (500, 4, (128, 1)), (256, 4, (64, 1)), (1024, 4, (256, 1)), (128, 4, (128, 1)),
+          (6, 2, (128, 1)), (50, 2, (32, 1)), (126, 2, (64, 1)), (250, 2, (128, 1)), (128, 2, (64, 1)),
+          (300, 4, (64, 1)), (500, 4, (64, 1)), (1000, 4, (128, 1)), (250, 2, (64, 1)), (1, 1, (7, 3)),
+          (37, 1, (128, 1)), (64, 2, (32, 4)), (16, 4, (4, 32))]
+# steps of FP32 arithmetic on deviations of order 0.1: 5 x 16 roundings of 2^-24; one unit of binary16 or
+# bfloat16 at 0.1 where a rounding falls the other way, carried through 5 steps
+TOLERANCE = {"f64": 1e-13, "f32": 5 * 16 * 2.0 ** -24 * 0.1, "f16dev": 4 * 2.0 ** -14, "bf16dev": 4 * 2.0 ** -11}
+
+
+@pytest.mark.parametrize("pattern", ["ab", "aa"])
+@pytest.mark.parametrize("store", ["f64", "f32", "f16dev"])
+@pytest.mark.parametrize("nx,V,block", SHAPES)
+def test_every_exchange_gives_the_state_of_the_scalar_path(nx, V, block, store, pattern):
+    if store == "f64" and V == 4:
+        pytest.skip("FP64 takes at most two sites per thread")
+    for ny, nz in ((1, 1), (5, 7), (3, 32)):
+        cfg = box(nx, ny, nz, store, pattern, kT=1e-3, gamma_ghost=0.2, force_amp=1e-3)
+        got = []
+        for launch in ((1, 64, 1), (V,) + block):
+            with flb.flb_create_ex(cfg) as ctx:
+                ctx.flb_set_launch(*launch)
+                ctx.flb_step(5)
+                got.append(ctx.flb_get_populations())
+        assert np.abs(got[0] - got[1]).max() <= TOLERANCE[store], (ny, nz)
+
+
+@pytest.mark.parametrize("pattern", ["ab", "aa"])
+@pytest.mark.parametrize("store", ["f64", "f32", "f16dev"])
+def test_batch_of_every_row_length_equals_the_boxes_alone(store, pattern):
+    edges = [(e, 3 + e % 5, 4) for e in (1, 2, 6, 12, 20, 28, 36, 40, 64, 100, 128, 132, 260, 516)]
+    for V in (1, 2, 4):
+        cfgs = [box(*(e if V == 1 else ((e[0] + V - 1) // V * V,) + e[1:]), store, pattern, kT=1e-3, replica=r)
+                for r, e in enumerate(edges)]
+        with flb.flb_create_batch(cfgs) as ctx:
+            ctx.flb_set_launch(2 if store == "f64" and V == 4 else V, 32, 4)
+            ctx.flb_step(5)
+            got = [ctx.flb_get_populations(b) for b in range(len(cfgs))]
+        for b, cfg in enumerate(cfgs):
+            with flb.flb_create_ex(cfg) as ctx:
+                ctx.flb_set_launch(1, 64, 1)
+                ctx.flb_step(5)
+                assert np.abs(ctx.flb_get_populations() - got[b]).max() <= TOLERANCE[store], (V, b)
+
+
+@pytest.mark.parametrize("nx", [8, 12, 13, 16, 24, 36, 48, 64, 72, 100, 125, 128, 160, 250, 256, 300, 400, 512, 1000])
+@pytest.mark.parametrize("store", ["f64", "f32", "f16dev"])
+def test_automatic_launch_fits_its_box_and_is_accepted_back(nx, store):
+    with flb.flb_create_ex(box(nx, 6, 4, store, "ab")) as ctx:
+        V, bx, by = ctx.flb_get_launch()
+        assert nx % V == 0 and 1 <= bx * by <= 256 and (V == 1 or bx * by % 32 == 0)
+        ctx.flb_step(2)
+        want = raw(ctx)
+    with flb.flb_create_ex(box(nx, 6, 4, store, "ab")) as ctx:
+        ctx.flb_set_launch(V, bx, by)
+        ctx.flb_step(2)
+        assert np.array_equal(raw(ctx), want)
