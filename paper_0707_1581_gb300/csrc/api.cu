@@ -252,15 +252,22 @@ void fill_consts(const flb_config &c, CollideConsts<R> &K)
         if (k == 4) g = c.gamma_bulk;
         else if (k >= 5 && k <= 9) g = c.gamma_shear;
         else if (k >= 10) g = c.gamma_ghost;
-        const double w = mode_norm(k);
+        // collide64 takes 1/36 with them, and its own signs and factors (see CollideConsts)
+        constexpr bool f64 = sizeof(R) == 8;
+        const double w = (f64 ? 36.0 : 1.0) * mode_norm(k);
         K.relax[k] = (R)(g / w);
-        K.eq[k] = (R)((1.0 - g) / w);
+        K.eq[k] = (R)((f64 && k == 5 ? g - 1.0 : 1.0 - g) / w);
         const bool thermal = k >= 4 && (k <= 9 || c.noise_ghosts);
-        const double var = mu * c.rho0 * w * (1.0 - g * g);
+        const double var = mu * c.rho0 * mode_norm(k) * (1.0 - g * g);
         // the FP32 Box-Muller returns normals / sqrt(2 ln 2); its amplitudes carry the factor
-        const double bm = sizeof(R) == 4 ? kBoxMullerF32Scale : 1.0;
+        const double bm = f64 ? 1.0 : kBoxMullerF32Scale;
         K.noise[k] = (R)(thermal && var > 0.0 ? bm * std::sqrt(var) / w : 0.0);
-        if (k < 10) K.forcing[k] = (R)((1.0 + g) / (2.0 * w));
+        if (k < 10) K.forcing[k] = (R)((f64 && k == 4 ? 2.0 : (f64 && k == 5 ? 4.0 : 1.0)) * (1.0 + g) / (2.0 * w));
+    }
+    if constexpr (sizeof(R) == 8) {
+        K.noise10 = -2.0 * K.noise[10];
+        K.noise16[0] = -4.0 * K.noise[16];
+        K.noise16[1] = 12.0 * K.noise[16];
     }
     K.force_amp = (R)c.force_amp;
     K.force_phase = (R)(2.0 / c.nz);

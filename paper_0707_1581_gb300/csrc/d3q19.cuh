@@ -63,6 +63,9 @@ __host__ __device__ constexpr double mode_norm(int k)
 //   relax[k] = gamma_k / w_k,  eq[k] = (1 - gamma_k) / w_k,
 //   noise[k] = sigma_k / w_k (times kBoxMullerF32Scale in FP32, see box_muller),
 //   forcing[k] = (1 + gamma_k) / (2 w_k)  (k = 4..9)
+// FP64 (collide64): all of them over 36, eq[5] with a minus sign, forcing[4] and
+// [5] times 2 and 4, and noise10 = -2 noise[10] (modes 10..12 have the same amplitude),
+// noise16 = -4, 12 times noise[16].
 // The 2^16 values each Box-Muller factor of the FP64 generator can take (its
 // uniforms have 16 bits): r[k] = sqrt(-2 ln u) and cs[k] = (cos, sin)(2 pi u)
 // at u = (k + 1/2) 2^-16.  Filled once per context by k_bm_tables with the
@@ -75,7 +78,7 @@ struct BoxMullerTables {
     const double2 *cs;
 };
 
-// Only the FP64 constants carry the tables (a base class, so that the FP32
+// Only the FP64 constants carry the tables and collide64's amplitudes (a base class, so that the FP32
 // constants keep the layout, and the kernels the constant loads, they had).
 template <class R>
 struct CollideTables {
@@ -83,6 +86,7 @@ struct CollideTables {
 template <>
 struct CollideTables<double> {
     BoxMullerTables bm;
+    double noise10, noise16[2];
 };
 __device__ __forceinline__ BoxMullerTables bm_of(const CollideTables<float> &) { return BoxMullerTables{nullptr, nullptr}; }
 __device__ __forceinline__ const BoxMullerTables &bm_of(const CollideTables<double> &K) { return K.bm; }
@@ -350,6 +354,15 @@ __device__ __forceinline__ void forward_modes(const R (&f)[Q], R (&m)[Q])
 // The collision of one site, in place on f[19], which holds the deviations
 // n_i - rho0 a_i (so m_0 = rho - rho0; modes k >= 1 equal those of n).
 //   Fx  = body force density of this site along x (used when FORCE).
+//
+// Two orders of the arithmetic.  collide (FP32, one site or a pair) takes about
+// 180 operations per site with gamma_ghost = 0.  collide64 takes about 150: FP64
+// kernels are bound by the FP64 unit (64 cycles per warp instruction on each SM
+// quarter), and 128^3 takes 677 us per step with it against 772.  FP32 keeps its
+// order although collide64's would give the 16-bit kernels 4-8 %: a stored value's
+// rounding to 16 bits follows the last FP32 bit, so another order gives another
+// (equally good) run -- the total momentum of a bfloat16 box differs in its second
+// digit after 20 steps -- and runs are to stay reproducible.
 // R = F2 collides two sites at once (site = their two indices; constants K
 // in FP32): the same operations, lane by lane.
 // --------------------------------------------------------------------------
@@ -495,6 +508,118 @@ __device__ __forceinline__ void collide(R (&f)[Q], const CollideConsts<KR> &K, S
         f[17] = fma_r(w2, Ozxm, e);
         f[18] = fma_r(-w2, Ozxm, e);
     }
+}
+
+template <int NOISE, bool FORCE, bool DRAWN>
+__device__ __forceinline__ void collide64(double (&f)[Q], const CollideConsts<double> &K, uint32_t site, uint32_t step,
+                                          uint32_t replica, double Fx, double (&g)[16])
+{
+    using R = double;
+    constexpr bool kin0 = NOISE == 2;
+    R m[Q];
+    forward_modes<R>(f, m);
+    const R m0 = m[0], jx = m[1], jy = m[2], jz = m[3], m4 = m[4], m5 = m[5], m6 = m[6], m7 = m[7], m8 = m[8];
+    const R m9 = m[9], m10 = m[10], m11 = m[11], m12 = m[12], m13 = m[13], m14 = m[14], m15 = m[15];
+    const R m16 = m[16], m17 = m[17], m18 = m[18];
+
+    // --- equilibrium stress modes of Eq. derived_equil_distrib ---
+    const R rho = K.rho0 + m0;
+    const R inv_rho = recip(rho);
+    const R px = FORCE ? fma_r(R(0.5), Fx, jx) : jx;       // rho u (half-step momentum)
+    const R ux = px * inv_rho, uy = jy * inv_rho, uz = jz * inv_rho;
+    const R exx = px * ux, ezz = jz * uz, eyz = fma_r(jy, uy, ezz);
+    const R eq4 = exx + eyz;                               // rho u^2
+    const R eq5 = fma_r(R(-2), exx, eyz);                  // -rho (3 ux^2 - u^2); K.eq[5] carries the sign
+    const R eq6 = fma_r(jy, uy, -ezz);                     // rho (uy^2 - uz^2)
+    const R eq7 = px * uy, eq8 = jy * uz, eq9 = jz * ux;   // rho u_a u_b
+
+    // --- relaxation (+ noise, + forcing), scaled by 1/(36 w_k) for the inverse ---
+    const R w = R(1.0 / 36.0);
+    const R t0 = w * m0;
+    const R w3 = R(1.0 / 12.0);
+    const R t1 = w3 * (FORCE ? jx + Fx : jx), t2 = w3 * jy, t3 = w3 * jz;
+    R t4 = fma_r(K.relax[4], m4, K.eq[4] * eq4);
+    R t5 = fma_r(K.relax[5], m5, K.eq[5] * eq5);
+    R t6 = fma_r(K.relax[6], m6, K.eq[6] * eq6);
+    R t7 = fma_r(K.relax[7], m7, K.eq[7] * eq7);
+    R t8 = fma_r(K.relax[8], m8, K.eq[8] * eq8);
+    R t9 = fma_r(K.relax[9], m9, K.eq[9] * eq9);
+    if (FORCE) {
+        // source S = uF + Fu of the second moment, F = (Fx, 0, 0): (1 + gamma_k) / 2
+        // times 2 uF, 4 uF, uy F and uz F in modes 4, 5, 7 and 9
+        const R uF = ux * Fx;
+        t4 = fma_r(K.forcing[4], uF, t4);
+        t5 = fma_r(K.forcing[5], uF, t5);
+        t7 = fma_r(K.forcing[7], uy * Fx, t7);
+        t9 = fma_r(K.forcing[9], uz * Fx, t9);
+    }
+    if (NOISE) {
+        if constexpr (!DRAWN) draw_normals<R>(K, site, step, replica, g);
+        if (K.noise_rho_local) {
+            // variance mu rho w_k with the local density
+            const R scale = sqrt_r(rho * K.inv_rho0);
+#pragma unroll
+            for (int k = 0; k < 15; ++k) g[k] *= scale;
+        }
+        t4 = fma_r(K.noise[4], g[0], t4);
+        t5 = fma_r(K.noise[5], g[1], t5);
+        t6 = fma_r(K.noise[6], g[2], t6);
+        t7 = fma_r(K.noise[7], g[3], t7);
+        t8 = fma_r(K.noise[8], g[4], t8);
+        t9 = fma_r(K.noise[9], g[5], t9);
+    }
+    // t_k of the kinetic modes 10..18.  With gamma_ghost = 0 they are only noise
+    // and are never formed: every use is a multiply-add of the normal.
+    R t[Q];
+    if constexpr (!kin0) {
+        const R m[Q] = {m0, jx, jy, jz, m4, m5, m6, m7, m8, m9, m10, m11, m12, m13, m14, m15, m16, m17, m18};
+#pragma unroll
+        for (int k = 10; k < Q; ++k) {
+            t[k] = K.relax[k] * m[k];
+            if (NOISE) t[k] = fma_r(K.noise[k], g[k - 4], t[k]);
+        }
+    }
+    // base + t_k, base - t_k and base + C t_k (Cn = C times the noise amplitude)
+    auto plus = [&](R base, int k) { return kin0 ? fma_r(K.noise[k], g[k - 4], base) : base + t[k]; };
+    auto minus = [&](R base, int k) { return kin0 ? fma_r(-K.noise[k], g[k - 4], base) : base - t[k]; };
+    auto times = [&](R base, int k, R C, R Cn) { return kin0 ? fma_r(Cn, g[k - 4], base) : fma_r(C, t[k], base); };
+
+    // --- inverse transform n*_i = a_i sum_k e_ki t_k, per opposite pair: the sums
+    // are n* / 36 for the diagonal velocities, twice that along the axes, 12
+    // times at rest ---
+    const R D = plus(t0 + t4, 16);
+    const R X2 = times(R(2.0 / 36.0) * m0, 16, R(-4), K.noise16[0]);      // 2 (t0 - 2 t16)
+    f[0] = fma_r(R(12), t0 - t4, kin0 ? K.noise16[1] * g[12] : R(12) * t[16]);
+    const R Pp = plus(t5, 17), Pm = minus(t5, 17), Rp = plus(t6, 18), Rm = minus(t6, 18);
+    const R Y2 = fma_r(R(-2), Pm, X2);
+    const R Ex2 = fma_r(R(4), Pm, X2), Ey2 = fma_r(R(2), Rm, Y2), Ez2 = fma_r(R(-2), Rm, Y2);
+    const R DP = D + Pp;
+    const R Exy = DP + Rp, Ezx = DP - Rp, Eyz = fma_r(R(-2), Pp, D);
+    const R Ox = times(t1, 10, R(-2), K.noise10), Oy = times(t2, 11, R(-2), K.noise10);
+    const R Oz = times(t3, 12, R(-2), K.noise10);
+    const R U1 = plus(t1, 10), U2 = plus(t2, 11), U3 = plus(t3, 12);
+    // odd parts of the diagonal pairs: (U1 +- U2) + (t13 -+ t14) = (U1 + t13) +-
+    // (U2 - t14), and the same in the other two planes
+    const R xy1 = plus(U1, 13), xy2 = minus(U2, 14);
+    const R yz1 = plus(U2, 14), yz2 = minus(U3, 15);
+    const R zx1 = plus(U3, 15), zx2 = minus(U1, 13);
+
+    f[1] = fma_r(R(2), Ox, Ex2);
+    f[2] = fma_r(R(-2), Ox, Ex2);
+    f[3] = fma_r(R(2), Oy, Ey2);
+    f[4] = fma_r(R(-2), Oy, Ey2);
+    f[5] = fma_r(R(2), Oz, Ez2);
+    f[6] = fma_r(R(-2), Oz, Ez2);
+    auto pair = [&](int i, R e, R o) {
+        f[i] = e + o;
+        f[i + 1] = e - o;
+    };
+    pair(7, Exy + t7, xy1 + xy2);
+    pair(9, Exy - t7, xy1 - xy2);
+    pair(11, Eyz + t8, yz1 + yz2);
+    pair(13, Eyz - t8, yz1 - yz2);
+    pair(15, Ezx + t9, zx1 + zx2);
+    pair(17, Ezx - t9, zx1 - zx2);
 }
 
 // --------------------------------------------------------------------------

@@ -107,7 +107,8 @@ __device__ __forceinline__ void update_sites(const BoxStep<S> &B, int x0, int y,
             f[i] = Storage<S>::load(load_ro(FLB_GUARD_LD(B, p, 1)));
         }
         if constexpr (kStart<S, V> == kAfterLoads) let_next_step_start();
-        collide<R, NOISE, FORCE, true>(f, B.K, site_row + (uint32_t)x, step, B.replica, Fx, g);
+        if constexpr (sizeof(R) == 8) collide64<NOISE, FORCE, true>(f, B.K, site_row + (uint32_t)x, step, B.replica, Fx, g);
+        else collide<R, NOISE, FORCE, true>(f, B.K, site_row + (uint32_t)x, step, B.replica, Fx, g);
         stochastic_round<S>(f, site_row + (uint32_t)x, step, B.replica, B.K.rk0, B.K.rk1);
         if constexpr (kStart<S, V> == kBeforeStores) let_next_step_start();
 #pragma unroll
@@ -479,8 +480,12 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
         }
     } else {
 #pragma unroll
-        for (int v = 0; v < V; ++v)
-            collide<R, NOISE, FORCE, kDrawn>(f[v], B.K, site0 + v, step, B.replica, Fx, g[kDrawn ? v : 0]);
+        for (int v = 0; v < V; ++v) {
+            if constexpr (sizeof(R) == 8)
+                collide64<NOISE, FORCE, kDrawn>(f[v], B.K, site0 + v, step, B.replica, Fx, g[kDrawn ? v : 0]);
+            else
+                collide<R, NOISE, FORCE, kDrawn>(f[v], B.K, site0 + v, step, B.replica, Fx, g[kDrawn ? v : 0]);
+        }
     }
 #pragma unroll
     for (int v = 0; v < V; ++v) stochastic_round<S>(f[v], site0 + v, step, B.replica, B.K.rk0, B.K.rk1);
