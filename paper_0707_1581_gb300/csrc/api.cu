@@ -19,6 +19,7 @@
 #include "d2q9.cuh"
 #include "diag_kernels.cuh"
 #include "kernels.cuh"
+#include "profile.cuh"
 
 using namespace flb;
 
@@ -104,6 +105,8 @@ struct flb_ctx {
     bool kin0 = true;               // every box has gamma_ghost = 0
     double *d_scratch = nullptr;    // canonical gather / moments staging
     size_t scratch_bytes = 0;
+    void *h_result = nullptr;       // page-locked memory that small results are written to
+    size_t h_result_bytes = 0;
     // host-resident stepping: copy streams and per-chunk events
     cudaStream_t s_up = nullptr, s_down = nullptr;
     std::vector<cudaEvent_t> ev_up, ev_comp;
@@ -524,6 +527,24 @@ int ensure_scratch(flb_ctx *c, size_t bytes)
     }
     c->scratch_bytes = bytes;
     return FLB_OK;
+}
+
+// Page-locked host memory of the context for a result of `bytes`, which a kernel
+// can write itself; NULL if the system has none to give.
+void *result_memory(flb_ctx *c, size_t bytes)
+{
+    if (c->h_result_bytes < bytes) {
+        if (c->h_result) cudaFreeHost(c->h_result);
+        c->h_result = nullptr;
+        c->h_result_bytes = 0;
+        if (cudaMallocHost(&c->h_result, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            c->h_result = nullptr;
+            return nullptr;
+        }
+        c->h_result_bytes = bytes;
+    }
+    return c->h_result;
 }
 
 // Slab units (z-planes or y-rows) per slab so that `per_site` doubles per site fit in 256 MiB.
@@ -966,14 +987,26 @@ int create_impl(const flb_config *cfgs, int nboxes, flb_ctx **out)
     return FLB_OK;
 }
 
-template <class S>
-cudaError_t z_profile_t(flb_ctx *c, const Box &b, double *out)
+cudaError_t profile_box(flb_ctx *c, const Box &b, double *part, double *out)
 {
-    if (is_d2(c))
-        return d2::launch_y_profile<S>(static_cast<const S *>(state_buf(c, b)), b.plane, layout_of(c, c->step),
-                                       b.cfg.nx, b.cfg.ny, b.cfg.rho0, out, c->stream);
-    return launch_z_profile<S>(static_cast<const S *>(state_buf(c, b)), b.plane, layout_of(c, c->step), b.cfg.nx,
-                               b.cfg.ny, b.cfg.nz, b.cfg.rho0, out, c->stream);
+    const bool two = is_d2(c);
+    const int layout = layout_of(c, c->step), n = units(b);
+    const int64_t M = unit_sites(b);
+    const void *buf = state_buf(c, b);
+    switch (c->store) {
+    case FLB_STORE_F64:
+        return launch_profile<double>(static_cast<const double *>(buf), b.plane, layout, M, n, two, b.cfg.rho0, part, out,
+                                      c->stream);
+    case FLB_STORE_F32:
+        return launch_profile<float>(static_cast<const float *>(buf), b.plane, layout, M, n, two, b.cfg.rho0, part, out,
+                                     c->stream);
+    case FLB_STORE_F16DEV:
+        return launch_profile<__half>(static_cast<const __half *>(buf), b.plane, layout, M, n, two, b.cfg.rho0, part, out,
+                                      c->stream);
+    default:   // both bfloat16 formats hold the same bits
+        return launch_profile<__nv_bfloat16>(static_cast<const __nv_bfloat16 *>(buf), b.plane, layout, M, n, two,
+                                             b.cfg.rho0, part, out, c->stream);
+    }
 }
 
 Box *box_of(flb_ctx *c, int box)
@@ -1051,6 +1084,7 @@ void flb_destroy(flb_ctx *c)
     for (Box &b : c->boxes) free_box(c, b);
     dev_free(c, c->d_step);
     dev_free(c, c->d_scratch);
+    if (c->h_result) cudaFreeHost(c->h_result);
     dev_free(c, c->d_bm);
     dev_free(c, c->d_viol);
     for (cudaEvent_t e : c->ev_up) cudaEventDestroy(e);
@@ -1345,19 +1379,19 @@ int flb_box_z_profile(flb_ctx *c, int box, double *rho, double *j)
     Box *b = box_of(c, box);
     if (!b) return fail(c, FLB_EINVAL, "bad box index");
     const int nz = units(*b);            // z-planes, or y-rows of a D2Q9 box
-    int rc = ensure_scratch(c, (size_t)4 * nz * sizeof(double));
+    const size_t part = (size_t)b->Q * nz * profile_chunks(unit_sites(*b), nz, b->Q), means = 4 * (size_t)nz;
+    int rc = ensure_scratch(c, (part + means) * sizeof(double));
     if (rc) return rc;
-    cudaError_t e;
-    switch (c->store) {
-    case FLB_STORE_F64: e = z_profile_t<double>(c, *b, c->d_scratch); break;
-    case FLB_STORE_F32: e = z_profile_t<float>(c, *b, c->d_scratch); break;
-    case FLB_STORE_F16DEV: e = z_profile_t<__half>(c, *b, c->d_scratch); break;
-    case FLB_STORE_BF16SR: e = z_profile_t<bf16sr>(c, *b, c->d_scratch); break;
-    default: e = z_profile_t<__nv_bfloat16>(c, *b, c->d_scratch); break;
+    // the means are written straight to page-locked memory where there is some
+    std::vector<double> own;
+    double *h = static_cast<double *>(result_memory(c, means * sizeof(double)));
+    double *out = h ? h : c->d_scratch + part;
+    CK(c, profile_box(c, *b, c->d_scratch, out));
+    if (!h) {
+        own.resize(means);
+        h = own.data();
+        CK(c, cudaMemcpyAsync(h, out, means * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     }
-    CK(c, e);
-    std::vector<double> h(4 * (size_t)nz);
-    CK(c, cudaMemcpyAsync(h.data(), c->d_scratch, h.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
     for (int z = 0; z < nz; ++z) {
         if (rho) rho[z] = h[z];

@@ -115,14 +115,6 @@ cudaError_t launch_stats_partial(const S *buf, int64_t plane, int layout, int nx
 }
 
 template <class S>
-cudaError_t launch_y_profile(const S *buf, int64_t plane, int layout, int nx, int ny, double rho0, double *out,
-                             cudaStream_t st)
-{
-    k_y_profile<S><<<ny, 256, 0, st>>>(buf, plane, layout, nx, ny, rho0, out);
-    return cudaGetLastError();
-}
-
-template <class S>
 cudaError_t launch_density(const S *buf, int64_t plane, int layout, int nx, int ny, typename Storage<S>::R *field,
                            cudaStream_t st)
 {
@@ -183,7 +175,6 @@ cudaError_t launch_moments(const double *n, int64_t slab, int nx, int ny, int y0
                                                     cudaStream_t);                                                  \
     template cudaError_t launch_stats_partial<S>(const S *, int64_t, int, int, int, double, double *, int,         \
                                                  cudaStream_t);                                                     \
-    template cudaError_t launch_y_profile<S>(const S *, int64_t, int, int, int, double, double *, cudaStream_t);   \
     template cudaError_t launch_density<S>(const S *, int64_t, int, int, int, typename Storage<S>::R *, cudaStream_t);
 
 FLB_D2_INSTANTIATE(double)

@@ -1,6 +1,6 @@
 // d2q9_diag.cuh -- the D2Q9 kernels outside the time step: gather and scatter
 // of canonical populations, the equilibrium initialisation, the statistics
-// pass, row profiles and the density field of S(q) (Table I lattice, the same
+// pass and the density field of S(q) (Table I lattice, the same
 // conventions as the D3Q19 diagnostics).
 #pragma once
 
@@ -255,44 +255,6 @@ __global__ void __launch_bounds__(256) k_stats_partial(const S *__restrict__ buf
         double v = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += wsum[w][threadIdx.x];
         partial[(int64_t)blockIdx.x * W + threadIdx.x] = v;
-    }
-}
-
-// Row means of rho and j along y: one block per row.  out[y] = <rho>,
-// out[ny + 3 y + a] = <j_a> (a = 0, 1; the third entry is 0).
-template <class S>
-__global__ void __launch_bounds__(256) k_y_profile(const S *__restrict__ buf, int64_t plane, int layout, int nx, int ny,
-                                                   double rho0, double *__restrict__ out)
-{
-    const int y = blockIdx.x;
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const Slot2 sl = canonical_slot(layout, i, x, y, nx, ny);
-            const double v = Storage<S>::to_double(buf[(int64_t)sl.q * plane + sl.y * nx + sl.x]) + rho0 * weight(i);
-            acc[0] += v;
-            acc[1] += vel_x(i) * v;
-            acc[2] += vel_y(i) * v;
-        }
-    }
-    __shared__ double red[3][8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        double v = acc[k];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if (lane == 0) red[k][warp] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 4) {
-        double v = 0.0;
-        if (threadIdx.x < 3)
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
-        v /= (double)nx;
-        if (threadIdx.x == 0) out[y] = v;
-        else out[ny + 3 * y + threadIdx.x - 1] = v;
     }
 }
 

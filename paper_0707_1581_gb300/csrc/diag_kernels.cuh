@@ -1,7 +1,7 @@
 // diag_kernels.cuh -- D3Q19 kernels outside the time step, templated on the
 // storage format S: canonical gather/scatter of the populations, the rest or
-// velocity-field initialisation, the per-block statistics pass, plane profiles
-// and the density field of S(q); with their launch wrappers.  The
+// velocity-field initialisation and the per-block statistics pass; with their
+// launch wrappers.  The
 // step_<format>.cu files instantiate them (FLB_INSTANTIATE).
 #pragma once
 
@@ -395,48 +395,6 @@ __global__ void __launch_bounds__(256) k_stats_partial_batch(const __grid_consta
     stats_pass<S>(B.buf, B.plane, layout, B.nx, B.ny, B.nz, B.rho0, B.partial, b - B.block0, B.nblocks, B.rho_out);
 }
 
-// Means over each z-plane of rho and j = sum_i n_i c_i (FP64 sums of the
-// stored values): one block per plane.  out[z] = <rho>, out[nz + 3 z + a] = <j_a>.
-template <class S>
-__global__ void __launch_bounds__(256) k_z_profile(const S *__restrict__ buf, int64_t plane, int layout, int nx, int ny,
-                                                   int nz, double rho0, double *__restrict__ out)
-{
-    const int z = blockIdx.x;
-    const int nxy = nx * ny;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int s = threadIdx.x; s < nxy; s += blockDim.x) {
-        const int x = s % nx, y = s / nx;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const Slot sl = canonical_slot(layout, i, x, y, z, nx, ny, nz);
-            double v = Storage<S>::to_double(buf[(int64_t)sl.q * plane + ((int64_t)sl.z * ny + sl.y) * nx + sl.x]);
-            if (Storage<S>::dev) v += rho0 * weight(i);
-            acc[0] += v;
-            acc[1] += vel_x(i) * v;
-            acc[2] += vel_y(i) * v;
-            acc[3] += vel_z(i) * v;
-        }
-    }
-    __shared__ double red[4][8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        double v = acc[k];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if (lane == 0) red[k][warp] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 4) {
-        double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
-        v /= (double)nxy;
-        if (threadIdx.x == 0) out[z] = v;
-        else out[nz + 3 * z + threadIdx.x - 1] = v;
-    }
-}
-
-// rho(r) - rho0 of the canonical state as a complex FP64 field (for S(q)).
 // Sums nblocks partials (fixed order) and adds them to acc[kStatWidth];
 // also records the first and last total mass and momentum of the samples
 // (acc layout described in internal.h).
@@ -494,14 +452,5 @@ cudaError_t launch_stats_partial_batch(const StatsTable<S> &T, int total_blocks,
     k_stats_partial_batch<S><<<total_blocks, 256, 0, st>>>(T, layout);
     return cudaGetLastError();
 }
-
-template <class S>
-cudaError_t launch_z_profile(const S *buf, int64_t plane, int layout, int nx, int ny, int nz, double rho0, double *out,
-                             cudaStream_t st)
-{
-    k_z_profile<S><<<nz, 256, 0, st>>>(buf, plane, layout, nx, ny, nz, rho0, out);
-    return cudaGetLastError();
-}
-
 
 }  // namespace flb

@@ -139,10 +139,6 @@ cudaError_t launch_relayout(const void *src, int from, void *dst, int to, size_t
                             int nz, bool d2, cudaStream_t st);
 cudaError_t launch_set_step(uint32_t *step_ptr, uint32_t value, cudaStream_t st);
 
-template <class S>
-cudaError_t launch_z_profile(const S *buf, int64_t plane, int layout, int nx, int ny, int nz, double rho0, double *out,
-                             cudaStream_t st);
-
 // Static structure factor (sq.cu).  The density deviation rho - rho0 of a box
 // (written by the statistics pass, or for D2Q9 by d2::launch_density) in the
 // transform type (FP64 for the FP64 format, else FP32) is transformed to its
@@ -205,9 +201,6 @@ cudaError_t launch_init_equilibrium(S *buf, int64_t plane, int layout, int nx, i
 template <class S>
 cudaError_t launch_stats_partial(const S *buf, int64_t plane, int layout, int nx, int ny, double rho0,
                                  double *partial, int nblocks, cudaStream_t st);
-template <class S>
-cudaError_t launch_y_profile(const S *buf, int64_t plane, int layout, int nx, int ny, double rho0, double *out,
-                             cudaStream_t st);
 template <class S>
 cudaError_t launch_density(const S *buf, int64_t plane, int layout, int nx, int ny, typename Storage<S>::R *field,
                            cudaStream_t st);

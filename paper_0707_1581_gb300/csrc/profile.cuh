@@ -1,0 +1,207 @@
+// profile.cuh -- plane averages of the canonical state (flb_box_z_profile) for
+// both lattices.
+//
+// A unit is a z-plane of a D3Q19 box or a row y of a D2Q9 box.  The shifts of
+// a population inside its unit do not change the unit's sum, so the sum of the
+// canonical n_i over unit u is the sum of one slot's contiguous unit u - c_i: the
+// first kernel sums every unit of every slot as one stream, the second combines
+// the Q sums of each unit.  Bound by HBM: 512^3 FP32 1.42 ms per call (10.2 GB at
+// 7.2 TB/s), 256^3 bfloat16 0.13 ms; one block per plane with every site's
+// populations added in FP64 took 34.3 and 4.3 ms, 64^3 FP32 160 us (now 28, of
+// which about 20 are the call's launches and wait).
+#pragma once
+
+#include "d3q19.cuh"
+#include "internal.h"
+
+namespace flb {
+namespace profile {
+
+// s + v without a rounding error: the sum and what it lost (Knuth's TwoSum).
+__device__ __forceinline__ float two_sum(float a, float b, float &err)
+{
+    const float s = __fadd_rn(a, b), bb = __fadd_rn(s, -a);
+    err = __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb));
+    return s;
+}
+
+// A running sum of 16- or 32-bit values as an unevaluated pair of floats (48
+// bits): an FP64 addition occupies an SM quarter's FP64 unit for 64 cycles per
+// warp, and a conversion to FP64 as long, seven FP32 additions for seven.  A
+// sum that leaves the range of FP32 (or meets an infinity or NaN) shows as a
+// non-finite hi; its values are then summed again in FP64.
+struct PairSum {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v)
+    {
+        float e;
+        hi = two_sum(hi, v, e);
+        lo += e;
+    }
+    __device__ __forceinline__ void add(PairSum o)
+    {
+        add(o.hi);
+        lo += o.lo;
+    }
+};
+
+constexpr int kThreads = 256;     // per block
+constexpr int kUnroll = 4;        // 16-byte loads in flight per thread
+
+// T threads (a warp or the block) sum chunk c of `chunks` of unit u of slot q, M
+// elements per unit, into part[(q units + u) chunks + c]; work item w is (c, q, u)
+// with u fastest.
+template <class S, int T>
+__global__ void __launch_bounds__(kThreads) k_unit_sums(const S *__restrict__ buf, int64_t plane, int64_t M, int units,
+                                                        int64_t items, int chunks, double *__restrict__ part)
+{
+    constexpr int E = 16 / sizeof(S);   // elements per 16-byte load
+    constexpr int kWarps = T / 32;
+    const int tid = (int)threadIdx.x % T;
+    const int64_t w = (int64_t)blockIdx.x * (kThreads / T) + threadIdx.x / T;
+    if (w >= items) return;             // whole warps: T is 32 or the block
+    const int u = (int)(w % units);
+    const int64_t qc = w / units;
+    const int q = (int)(qc / chunks), c = (int)(qc % chunks);
+    const int64_t per = (M + chunks - 1) / chunks, c0 = c * per;
+    const int64_t n = max((int64_t)0, min(per, M - c0));
+    const S *p = buf + q * plane + u * M + c0;
+    // up to the first 16-byte boundary and behind the last one: single elements
+    const int64_t head = min(n, (int64_t)((16 - reinterpret_cast<uintptr_t>(p) % 16) % 16 / sizeof(S)));
+    const int64_t vecs = (n - head) / E, tail = n - head - vecs * E;
+    const uint4 *v = reinterpret_cast<const uint4 *>(p + head);
+    auto each = [&](auto f) {   // f(value, which of two chains)
+        if (tid < head) f(p[tid], 0);
+        if (tid < tail) f(p[head + vecs * E + tid], 1);
+        for (int64_t i0 = tid; i0 < vecs; i0 += kUnroll * T) {
+            uint4 x[kUnroll];
+#pragma unroll
+            for (int r = 0; r < kUnroll; ++r)
+                x[r] = i0 + r * T < vecs ? v[i0 + r * T] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int r = 0; r < kUnroll; ++r) {
+                const S *e = reinterpret_cast<const S *>(&x[r]);
+#pragma unroll
+                for (int k = 0; k < E; ++k) f(e[k], k & 1);
+            }
+        }
+    };
+    double sum;
+    if constexpr (sizeof(S) == 8) {
+        sum = 0.0;
+        each([&](S x, int) { sum += x; });
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    } else {
+        PairSum a, b;
+        each([&](S x, int k) {
+            if (k) b.add(Storage<S>::load(x));
+            else a.add(Storage<S>::load(x));
+        });
+        a.add(b);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            PairSum o;
+            o.hi = __shfl_xor_sync(0xffffffffu, a.hi, off);
+            o.lo = __shfl_xor_sync(0xffffffffu, a.lo, off);
+            a.add(o);
+        }
+        sum = (double)a.hi + (double)a.lo;
+        if (__any_sync(0xffffffffu, !isfinite(a.hi) || !isfinite(a.lo))) {
+            sum = 0.0;
+            each([&](S x, int) { sum += Storage<S>::to_double(x); });
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+        }
+    }
+    if constexpr (kWarps > 1) {
+        __shared__ double wsum[kWarps];
+        if ((tid & 31) == 0) wsum[tid >> 5] = sum;
+        __syncthreads();
+        sum = 0.0;
+        if (tid == 0) {
+#pragma unroll
+            for (int k = 0; k < kWarps; ++k) sum += wsum[k];
+        }
+    }
+    if (tid == 0) part[((int64_t)q * units + u) * chunks + c] = sum;
+}
+
+// Warp u: out[u] = rho0 + sum_i s_i / M, out[units + 3 u + a] = sum_i c_ia s_i / M,
+// s_i (lane i) the sum of the deviation n_i over unit u.  D2: the D2Q9 velocities
+// in rows y (the third component is 0).
+template <bool D2>
+__global__ void __launch_bounds__(128) k_unit_means(const double *__restrict__ part, int layout, int64_t M, int units,
+                                                    int chunks, double rho0, double *__restrict__ out)
+{
+    constexpr int NQ = D2 ? 9 : 19;
+    const int i = (int)threadIdx.x & 31, u = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (u >= units) return;   // whole warps
+    constexpr int vx[2][19] = {{0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1},
+                               {0, 1, -1, 0, 0, 1, -1, 1, -1}};
+    constexpr int vy[2][19] = {{0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 1, -1, 1, -1, 0, 0, 0, 0},
+                               {0, 0, 0, 1, -1, 1, -1, -1, 1}};
+    constexpr int vz[19] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, 1, -1};
+    int cx = 0, cy = 0, cz = 0;
+#pragma unroll
+    for (int k = 0; k < NQ; ++k)
+        if (i == k) {
+            cx = vx[D2][k];
+            cy = vy[D2][k];
+            cz = D2 ? 0 : vz[k];
+        }
+    double s = 0.0;
+    if (i < NQ) {
+        const int q = layout == kAAOdd && i ? ((i & 1) ? i + 1 : i - 1) : i;
+        const int from = layout == kAAEven ? u : wrap_add(u, -(D2 ? cy : cz), units);
+        const double *p = part + ((int64_t)q * units + from) * chunks;
+#pragma unroll 8
+        for (int c = 0; c < chunks; ++c) s += p[c];
+    }
+    // 0 * infinity is NaN, as in a sum over the sites
+    double t[4] = {s, cx * s, cy * s, cz * s};
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) t[a] += __shfl_xor_sync(0xffffffffu, t[a], off);
+    }
+    // lane a writes value a (FP64 divisions are slow: one per lane)
+    const double v = (i == 0 ? t[0] : (i == 1 ? t[1] : (i == 2 ? t[2] : t[3]))) / (double)M;
+    if (i == 0) out[u] = rho0 + v;
+    else if (i < 4) out[units + 3 * u + i - 1] = v;
+}
+
+}  // namespace profile
+
+// Chunks per unit: enough blocks to fill the GPU (about eight per SM of 152) as
+// long as a block has at least 4096 elements.
+inline int profile_chunks(int64_t M, int units, int nq)
+{
+    const int64_t slots = (int64_t)units * nq, want = (1216 + slots - 1) / slots, most = M / 4096;
+    return (int)(want < most ? want : (most < 1 ? 1 : most));
+}
+
+// The means of every unit of a box (d2: D2Q9): part is scratch of nq units
+// chunks doubles, out receives 4 units doubles.  Units of fewer than 2048
+// elements are summed by one warp each.
+template <class S>
+cudaError_t launch_profile(const S *buf, int64_t plane, int layout, int64_t M, int units, bool d2, double rho0,
+                           double *part, double *out, cudaStream_t st)
+{
+    const int nq = d2 ? 9 : Q, chunks = profile_chunks(M, units, nq);
+    const int64_t items = (int64_t)units * nq * chunks;
+    constexpr int T = profile::kThreads;
+    if (M < 2048)
+        profile::k_unit_sums<S, 32><<<(unsigned)((items + T / 32 - 1) / (T / 32)), T, 0, st>>>(buf, plane, M, units,
+                                                                                               items, chunks, part);
+    else
+        profile::k_unit_sums<S, T><<<(unsigned)items, T, 0, st>>>(buf, plane, M, units, items, chunks, part);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const int blocks = (units + 3) / 4;
+    if (d2) profile::k_unit_means<true><<<blocks, 128, 0, st>>>(part, layout, M, units, chunks, rho0, out);
+    else profile::k_unit_means<false><<<blocks, 128, 0, st>>>(part, layout, M, units, chunks, rho0, out);
+    return cudaGetLastError();
+}
+
+}  // namespace flb

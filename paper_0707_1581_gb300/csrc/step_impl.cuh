@@ -167,5 +167,4 @@ cudaError_t launch_step_batch(const BatchParams<S> &P, int total_blocks, int lay
     template cudaError_t launch_stats_partial<S>(const S *, int64_t, int, int, int, int, double, double *, int,    \
                                                  typename Storage<S>::R *, cudaStream_t);                           \
     template cudaError_t launch_stats_partial_batch<S>(const StatsTable<S> &, int, int, cudaStream_t);             \
-    template cudaError_t launch_z_profile<S>(const S *, int64_t, int, int, int, int, double, double *, cudaStream_t); \
     }

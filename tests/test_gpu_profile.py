@@ -1,0 +1,71 @@
+"""Plane and row averages (flb_box_z_profile) against sums of the canonical populations."""
+import numpy as np
+import pytest
+
+from paper_0707_1581_gb300 import flb
+from paper_0707_1581_gb300.inputs import relative_perturbation
+
+pytestmark = pytest.mark.gpu
+
+WX = {19: [0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1], 9: [0, 1, -1, 0, 0, 1, -1, 1, -1]}
+WY = {19: [0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 1, -1, 1, -1, 0, 0, 0, 0], 9: [0, 0, 0, 1, -1, 1, -1, -1, 1]}
+WZ = {19: [0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, 1, -1], 9: [0] * 9}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_0707_1581_gb300 import build as B
+    B.build()
+
+
+def reference(n, two):
+    """rho[units], j[3][units] of populations n[q, ..., x], summed over all but the unit axis in FP64."""
+    q = n.shape[0]
+    m = n.sum(2) / n.shape[2] if two else n.sum((2, 3)) / (n.shape[2] * n.shape[3])
+    with np.errstate(invalid="ignore"):
+        return m.sum(0), np.stack([(np.array(w[q])[:, None] * m).sum(0) for w in (WX, WY, WZ)])
+
+
+# units of odd length (misaligned for vector loads), of fewer elements than a warp and than a block's
+# threshold, and few large ones (several blocks per unit)
+BOXES = [(1, 1, 1), (3, 5, 7), (17, 3, 6), (45, 46, 9), (64, 64, 8), (61, 67, 5), (301, 211, 2), (256, 256, 1)]
+
+
+@pytest.mark.parametrize("steps", [0, 1, 2])
+@pytest.mark.parametrize("pattern", ["ab", "aa"])
+@pytest.mark.parametrize("store", ["f64", "f32", "f16dev", "bf16dev", "bf16sr"])
+def test_profile_is_the_mean_of_the_populations(store, pattern, steps):
+    for two in (False, True):
+        for nx, ny, nz in BOXES:
+            cfg = flb.config(nx, ny * nz if two else ny, 1 if two else nz, kT=1e-3, gamma_shear=0.3, seed=2, store=store,
+                             pattern=pattern, lattice="d2q9" if two else "d3q19")
+            with flb.flb_create_ex(cfg) as ctx:
+                ctx.flb_step(steps)
+                rho, j = ctx.flb_z_profile()
+                want_rho, want_j = reference(ctx.flb_get_populations(), two)
+            # both sides round in FP64 (or 48 bits, of the small deviations): 1e-15 per unit of rho
+            assert np.abs(rho - want_rho).max() <= 2e-14 and np.abs(j - want_j).max() <= 2e-14, (two, nx, ny, nz)
+
+
+@pytest.mark.parametrize("store", ["f64", "f32", "f16dev"])
+def test_profile_of_values_beyond_the_ordinary(store):
+    """Sums beyond FP32's range stay finite; an infinity or NaN shows in its plane and nowhere else."""
+    shape = (19, 4, 40, 64)
+    big = {"f64": 1e300, "f32": 2e38, "f16dev": 6e4}[store]
+    with flb.flb_create_ex(flb.config(64, 40, 4, store=store, pattern="aa")) as ctx:
+        n = relative_perturbation(shape[1:], seed=3, amp=0.02) / 19
+        n[3, 1] = big
+        ctx.flb_set_populations(n)
+        n = ctx.flb_get_populations()
+        rho, j = ctx.flb_z_profile()
+        want_rho, want_j = reference(n, False)
+        assert np.isfinite(rho).all() and np.allclose(rho, want_rho, rtol=1e-12) and np.allclose(j, want_j, rtol=1e-12, atol=1e-13)
+        for bad in (np.inf, -np.inf, np.nan):
+            m = relative_perturbation(shape[1:], seed=3, amp=0.02) / 19
+            m[5, 2, 7, 9] = bad
+            ctx.flb_set_populations(m)
+            rho, j = ctx.flb_z_profile()
+            with np.errstate(invalid="ignore"):
+                want_rho, want_j = reference(ctx.flb_get_populations(), False)
+            assert np.array_equal(np.isnan(rho), np.isnan(want_rho)) and np.array_equal(np.isinf(rho), np.isinf(want_rho))
+            assert np.array_equal(np.isnan(j), np.isnan(want_j)) and np.array_equal(np.isinf(j), np.isinf(want_j))
