@@ -13,12 +13,16 @@
 #include <sys/mman.h>
 #include <unistd.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 #include <map>
 #include <mutex>
+#include <thread>
+#include <vector>
 
 #include "flb.h"
+#include "internal.h"
 
 namespace {
 
@@ -44,6 +48,50 @@ size_t huge_page_size()
 size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
+
+namespace flb {
+
+// A fresh result array has no pages yet, and a copy engine that meets them one
+// fault at a time writes at about 1 GB/s (GB300, 64 KB pages: 272 ms for the 319
+// MB of a 128^3 box's populations; 1.8 ms into memory that has its pages).  The
+// kernel is asked for all of them first (MADV_POPULATE_WRITE, which leaves the
+// contents alone), by a few threads, while the GPU works on what will be copied.
+// Best effort: where it fails the copy faults the pages in as before.
+void prefault(void *p, size_t bytes)
+{
+#ifndef MADV_POPULATE_WRITE
+    constexpr int MADV_POPULATE_WRITE = 23;   // Linux 5.14
+#endif
+    constexpr size_t kLeast = size_t(1) << 20, kPerThread = size_t(16) << 20;
+    if (!p || bytes < kLeast) return;
+    const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
+    // whole pages inside the array
+    const uintptr_t a = ((uintptr_t)p + page - 1) / page * page, b = ((uintptr_t)p + bytes) / page * page;
+    if (b <= a) return;
+    // nothing to do when a spread of its pages is there (asking anyway takes 1.5 ms for 319 MB)
+    bool resident = true;
+    for (int k = 0; k < 32 && resident; ++k) {
+        unsigned char in = 0;
+        const uintptr_t at = a + ((b - a) / page - 1) * k / 31 * page;
+        resident = mincore((void *)at, page, &in) == 0 && (in & 1);
+    }
+    if (resident) return;
+    const size_t n = std::max<size_t>(1, std::min<size_t>({8, (b - a) / kPerThread, std::thread::hardware_concurrency()}));
+    const uintptr_t step = ((b - a) / n + page - 1) / page * page;
+    auto part = [=](size_t k) {
+        const uintptr_t from = a + k * step, to = std::min(b, from + step);
+        if (from < to) (void)madvise((void *)from, to - from, MADV_POPULATE_WRITE);
+    };
+    std::vector<std::thread> others;
+    try {
+        for (size_t k = 1; k < n; ++k) others.emplace_back(part, k);
+    } catch (...) {   // no more threads: their parts stay for the copy
+    }
+    part(0);
+    for (std::thread &t : others) t.join();
+}
+
+}  // namespace flb
 
 extern "C" {
 

@@ -35,6 +35,9 @@ struct Launch {
     bool edgerow = false;   // blocks of one row each, scalar accesses at row and warp ends
 };
 
+// Gives the pages of a host array that is about to be overwritten (host_mem.cu).
+void prefault(void *p, size_t bytes);
+
 // Launches a step kernel with programmatic stream serialization: its blocks may
 // start once every block of the kernel before it has called
 // let_next_step_start (a kernel that never does is waited for as usual), and it
