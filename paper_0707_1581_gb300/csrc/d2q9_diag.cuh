@@ -5,6 +5,7 @@
 #pragma once
 
 #include "d2q9.cuh"
+#include "diag_kernels.cuh"
 
 namespace flb {
 namespace d2 {
@@ -102,6 +103,7 @@ __global__ void __launch_bounds__(256) k_stats_partial(const S *__restrict__ buf
 {
     // As the D3Q19 pass: R partials of 16 sites per lane, summed across the
     // warp at block-uniform points into per-warp FP64 rows (fixed orders).
+    let_next_step_start();
     using R = typename Storage<S>::R;
     constexpr int W = 27, kWarps = 8;
     __shared__ double wsum[kWarps][W];
@@ -113,15 +115,11 @@ __global__ void __launch_bounds__(256) k_stats_partial(const S *__restrict__ buf
 #pragma unroll
     for (int k = 0; k < W - 1; ++k) part[k] = R(0);
     unsigned sites_ok = 0, nonfinite = 0;
-    auto flush = [&]() {   // every lane of the warp calls it
+    auto flush = [&]() {   // every lane of the warp calls it (as the D3Q19 pass: lane k adds sum k)
+        const R v = warp_sums<R, W - 1>(part, lane);
+        if (lane < W - 1) wsum[warp][lane] += (double)v;
 #pragma unroll
-        for (int k = 0; k < W - 1; ++k) {
-            R v = part[k];
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-            if (lane == 0) wsum[warp][k] += (double)v;
-            part[k] = R(0);
-        }
+        for (int k = 0; k < W - 1; ++k) part[k] = R(0);
     };
     auto accumulate = [&](R (&d)[Q]) {
         bool finite = true;
@@ -241,6 +239,7 @@ __global__ void __launch_bounds__(256) k_stats_partial(const S *__restrict__ buf
         }
     }
     flush();
+    __syncwarp();
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         sites_ok += __shfl_xor_sync(0xffffffffu, sites_ok, off);

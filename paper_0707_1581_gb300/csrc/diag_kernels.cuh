@@ -147,6 +147,28 @@ struct StatsVec<8> {
     using T = uint2;
 };
 
+// The warp's sums of the lanes' N values v[0 .. N-1] (N <= 32): lane k returns the
+// sum of value k.  Five exchanges, each handing over the half of the values that
+// the partner lane keeps: 31 shuffles for up to 32 values, and every value is
+// added in the order of a butterfly over lane distances 16, 8, 4, 2, 1.
+template <class R, int N>
+__device__ __forceinline__ R warp_sums(const R (&v)[N], int lane)
+{
+    R w[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) w[k] = k < N ? v[k] : R(0);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const bool upper = (lane & off) != 0;   // keeps values off .. 2 off - 1 of the rest
+#pragma unroll
+        for (int k = 0; k < off; ++k) {
+            const R keep = upper ? w[k + off] : w[k], give = upper ? w[k] : w[k + off];
+            w[k] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
+    }
+    return w[0];
+}
+
 // Block `bid` of `nb` blocks of one box (blockDim.x <= 256, whole warps): its
 // rows' sums into row bid of partial.
 template <class S>
@@ -160,6 +182,7 @@ __device__ __forceinline__ void stats_pass(const S *__restrict__ buf, int64_t pl
     // order) and lane 0 adds the result to the warp's FP64 row in shared
     // memory, so FP64 arithmetic and the FP64 registers stay off the per-site
     // path.  Every order is fixed: the result is bitwise reproducible.
+    let_next_step_start();   // the pass over the partial sums (started as usual: it reads by the read-only path)
     using R = typename Storage<S>::R;
     constexpr int kWarps = 8;
     __shared__ double wsum[kWarps][kStatWidth];
@@ -170,15 +193,14 @@ __device__ __forceinline__ void stats_pass(const S *__restrict__ buf, int64_t pl
 #pragma unroll
     for (int k = 0; k < kStatWidth - 1; ++k) part[k] = R(0);
     unsigned sites_ok = 0, nonfinite = 0;
-    auto flush = [&]() {   // every lane of the warp calls it
+    // every lane of the warp calls it; lane k adds sum k in FP64: one conversion
+    // and one addition per flush for all 26 (each occupies an SM quarter's FP64
+    // unit for 64 cycles, so 26 of each by lane 0 took longer than the loads)
+    auto flush = [&]() {
+        const R v = warp_sums<R, kStatWidth - 1>(part, lane);
+        if (lane < kStatWidth - 1) wsum[warp][lane] += (double)v;
 #pragma unroll
-        for (int k = 0; k < kStatWidth - 1; ++k) {
-            R v = part[k];
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-            if (lane == 0) wsum[warp][k] += (double)v;
-            part[k] = R(0);
-        }
+        for (int k = 0; k < kStatWidth - 1; ++k) part[k] = R(0);
     };
     // returns rho - rho0 of the site (non-finite if a population is)
     auto accumulate = [&](R (&d)[Q]) -> R {
@@ -332,6 +354,7 @@ __device__ __forceinline__ void stats_pass(const S *__restrict__ buf, int64_t pl
         }
     }
     flush();
+    __syncwarp();
     // counts: sum of rho = sum of (rho - rho0) + rho0 per site; non-finite sites
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -398,7 +421,7 @@ __global__ void __launch_bounds__(256) k_stats_partial_batch(const __grid_consta
 // Sums nblocks partials (fixed order) and adds them to acc[kStatWidth];
 // also records the first and last total mass and momentum of the samples
 // (acc layout described in internal.h).
-__global__ void k_stats_finish(const double *__restrict__ partial, int nblocks, double *__restrict__ acc);
+__global__ void k_stats_finish(const double *partial, int nblocks, double *acc);
 
 
 template <class S>

@@ -38,12 +38,13 @@ struct Launch {
 // Gives the pages of a host array that is about to be overwritten (host_mem.cu).
 void prefault(void *p, size_t bytes);
 
-// Launches a step kernel with programmatic stream serialization: its blocks may
-// start once every block of the kernel before it has called
-// let_next_step_start (a kernel that never does is waited for as usual), and it
-// calls wait_for_previous_step before it touches the state.
+// Launches a kernel of the step or sampling chain with programmatic stream
+// serialization: its blocks may start once every block of the kernel before it has
+// called let_next_step_start (a kernel that never does is waited for as usual),
+// and it calls wait_for_previous_step before it touches what others write.
 template <class... KA, class... A>
-cudaError_t launch_chained(void (*kernel)(KA...), dim3 grid, dim3 block, cudaStream_t st, const A &...args)
+cudaError_t launch_chained_smem(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                const A &...args)
 {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -51,10 +52,16 @@ cudaError_t launch_chained(void (*kernel)(KA...), dim3 grid, dim3 block, cudaStr
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <class... KA, class... A>
+cudaError_t launch_chained(void (*kernel)(KA...), dim3 grid, dim3 block, cudaStream_t st, const A &...args)
+{
+    return launch_chained_smem(kernel, grid, block, 0, st, args...);
 }
 
 // The FP64 Box-Muller tables (BoxMullerTables): r[65536] then cs[65536] in one
