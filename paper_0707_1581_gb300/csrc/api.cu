@@ -1015,24 +1015,24 @@ Box *box_of(flb_ctx *c, int box)
     return &c->boxes[box];
 }
 
-// One chunk of planes [z0, z1) of the stream-collide kernel of box b.
+// One chunk of planes [z0, z1) of the stream-collide kernel of box b, at `step`.
 template <class S>
-cudaError_t step_chunk_t(flb_ctx *c, const Box &b, int orient, int layout, int z0, int z1)
+cudaError_t step_chunk_t(flb_ctx *c, const Box &b, int orient, int layout, uint64_t step, int z0, int z1)
 {
     BoxStep<S> s = make_step<S>(c, b, orient);
     s.z0 = z0;
     s.nzl = z1 - z0;
-    return launch_step<S>(s, layout, noise_mode(c), c->force, c->L, nullptr, (uint32_t)c->step, c->stream);
+    return launch_step<S>(s, layout, noise_mode(c), c->force, c->L, nullptr, (uint32_t)step, c->stream);
 }
 
-cudaError_t step_chunk(flb_ctx *c, const Box &b, int orient, int layout, int z0, int z1)
+cudaError_t step_chunk(flb_ctx *c, const Box &b, int orient, int layout, uint64_t step, int z0, int z1)
 {
     switch (c->store) {
-    case FLB_STORE_F64: return step_chunk_t<double>(c, b, orient, layout, z0, z1);
-    case FLB_STORE_F32: return step_chunk_t<float>(c, b, orient, layout, z0, z1);
-    case FLB_STORE_F16DEV: return step_chunk_t<__half>(c, b, orient, layout, z0, z1);
-    case FLB_STORE_BF16SR: return step_chunk_t<bf16sr>(c, b, orient, layout, z0, z1);
-    default: return step_chunk_t<__nv_bfloat16>(c, b, orient, layout, z0, z1);
+    case FLB_STORE_F64: return step_chunk_t<double>(c, b, orient, layout, step, z0, z1);
+    case FLB_STORE_F32: return step_chunk_t<float>(c, b, orient, layout, step, z0, z1);
+    case FLB_STORE_F16DEV: return step_chunk_t<__half>(c, b, orient, layout, step, z0, z1);
+    case FLB_STORE_BF16SR: return step_chunk_t<bf16sr>(c, b, orient, layout, step, z0, z1);
+    default: return step_chunk_t<__nv_bfloat16>(c, b, orient, layout, step, z0, z1);
     }
 }
 
@@ -1196,36 +1196,55 @@ int flb_box_step_host(flb_ctx *c, int box, void *host, int64_t nsteps)
         CK(c, cudaMemcpy2DAsync(src + off, pitch, h + off, pitch, w, Q19, cudaMemcpyHostToDevice, c->s_up));
         CK(c, cudaEventRecord(c->ev_up[k], c->s_up));
     }
-    for (int k = 0; k < K; ++k) {
-        if (local || K == 1) {
-            CK(c, cudaStreamWaitEvent(c->stream, c->ev_up[k], 0));
-        } else {
-            for (int d = -1; d <= 1; ++d) CK(c, cudaStreamWaitEvent(c->stream, c->ev_up[(k + d + K) % K], 0));
+    // Several steps of one box follow the uploads as a wave: step s (from 0) takes
+    // its j-th chunk, s + j (mod K), behind the chunk j + 2 of step s - 1, when the
+    // step before is done on that chunk and on both beside it, so the downloads
+    // start a few chunks behind the uploads and both copy directions run together
+    // (256^3 FP32, two steps: 8.5 ms, 13.2 with the downloads behind the last
+    // step).  More steps than an eighth of the chunks, and batches, whose other
+    // boxes take part in the further steps, step whole boxes.
+    const bool wave = nsteps > 1 && K >= 8 && nsteps - 1 <= K / 8 && c->boxes.size() == 1;
+    const int nwave = wave ? (int)nsteps : 1;
+    for (int tau = 0; tau < K + 2 * (nwave - 1); ++tau) {
+        for (int s = 0; s < nwave; ++s) {
+            const int j = tau - 2 * s;
+            if (j < 0 || j >= K) continue;
+            const int k = (s + j) % K;
+            if (s == 0) {
+                if (local || K == 1) {
+                    CK(c, cudaStreamWaitEvent(c->stream, c->ev_up[k], 0));
+                } else {
+                    for (int d = -1; d <= 1; ++d) CK(c, cudaStreamWaitEvent(c->stream, c->ev_up[(k + d + K) % K], 0));
+                }
+            }
+            const int o = c->pattern == FLB_PATTERN_AB ? orient ^ (s & 1) : orient;
+            CK(c, step_chunk(c, *b, o, layout_of(c, c->step + s), c->step + s, zb[k], zb[k + 1]));
+            if (s == nwave - 1) CK(c, cudaEventRecord(c->ev_comp[k], c->stream));
         }
-        CK(c, step_chunk(c, *b, orient, layout, zb[k], zb[k + 1]));
-        CK(c, cudaEventRecord(c->ev_comp[k], c->stream));
     }
-    if (c->pattern == FLB_PATTERN_AB) c->cur ^= 1;
-    c->step += 1;
+    const int last_layout = layout_of(c, c->step + nwave - 1);   // of the chunked step that downloads may follow
+    if (c->pattern == FLB_PATTERN_AB && (nwave & 1)) c->cur ^= 1;
+    c->step += nwave;
     // further steps on the device
-    for (int64_t left = nsteps - 1; left > 0; --left) {
+    const int64_t further = nsteps - nwave;
+    for (int64_t left = further; left > 0; --left) {
         CK(c, enqueue_one_step(c, c->cur, layout_of(c, c->step), nullptr, (uint32_t)c->step));
         if (c->pattern == FLB_PATTERN_AB) c->cur ^= 1;
         c->step += 1;
     }
     CK(c, cudaEventRecord(c->ev_done, c->stream));
-    // downloads: after one step a chunk is final once the computes that write
-    // it are done (its own; in the AA odd step also its neighbours'), so they
-    // are issued in the order the chunks become final (chunk 0 of an AA odd
-    // step waits for the last compute)
+    // downloads: after the last chunked step a chunk is final once the computes
+    // that write it are done (its own; in the AA odd step also its neighbours'), so
+    // they are issued in the order the chunks become final (the first chunk of an
+    // AA odd step waits for the last compute)
     char *dst = static_cast<char *>(state_buf(c, *b));
     std::vector<int> dorder(K);
-    for (int k = 0; k < K; ++k) dorder[k] = k;
-    if (nsteps == 1 && layout == kAAOdd && K > 1) std::rotate(dorder.begin(), dorder.begin() + 1, dorder.end());
+    for (int j = 0; j < K; ++j) dorder[j] = (nwave - 1 + j) % K;
+    if (further == 0 && last_layout == kAAOdd && K > 1) std::rotate(dorder.begin(), dorder.begin() + 1, dorder.end());
     for (int k : dorder) {
-        if (nsteps > 1) {
+        if (further > 0) {
             CK(c, cudaStreamWaitEvent(c->s_down, c->ev_done, 0));
-        } else if (layout == kAAOdd && K > 1) {
+        } else if (last_layout == kAAOdd && K > 1) {
             for (int d = -1; d <= 1; ++d) CK(c, cudaStreamWaitEvent(c->s_down, c->ev_comp[(k + d + K) % K], 0));
         } else {
             CK(c, cudaStreamWaitEvent(c->s_down, c->ev_comp[k], 0));

@@ -117,3 +117,25 @@ def test_automatic_launch_fits_its_box_and_is_accepted_back(nx, store):
         ctx.flb_set_launch(V, bx, by)
         ctx.flb_step(2)
         assert np.array_equal(raw(ctx), want)
+
+
+@pytest.mark.parametrize("nz,nsteps", [(8, 2), (9, 2), (31, 4), (32, 5), (40, 5), (40, 6), (7, 3)])
+@pytest.mark.parametrize("pattern,start", [("ab", 0), ("ab", 1), ("aa", 0), ("aa", 1)])
+def test_host_resident_steps_in_a_wave_equal_device_steps(pattern, start, nz, nsteps):
+    """Several steps per call, each a few chunks behind the one before (7 chunks and 6 steps of 32: whole boxes)."""
+    cfg = box(24, 6, nz, "f32", pattern, kT=1e-3, force_amp=1e-4)
+    with flb.flb_create_ex(cfg) as ref:
+        ref.flb_step(6 + start)
+        host = raw(ref)
+        ref.flb_step(nsteps)
+        want = raw(ref)
+        ref.flb_step(3)
+        later = raw(ref)
+    with flb.flb_create_ex(cfg) as ctx:
+        ctx.flb_step(6 + start)
+        ctx.flb_init_velocity(None)
+        ctx.flb_step_host(host, nsteps)
+        assert np.array_equal(host, want) and ctx.flb_get_step() == 6 + start + nsteps
+        assert np.array_equal(raw(ctx), want)
+        ctx.flb_step(3)
+        assert np.array_equal(raw(ctx), later)
