@@ -50,6 +50,7 @@ struct Box {
     CollideConsts<double> Kd;
     d2::CollideConsts<float> K2f;
     d2::CollideConsts<double> K2d;
+    void *d_fx = nullptr;           // body force per z-plane, compute type (D3Q19 with a force, not FP32)
     double *d_acc = nullptr;        // kAccWidth accumulators
     double *d_partial = nullptr;    // stats partials
     int stats_nb = 0;
@@ -344,6 +345,7 @@ BoxStep<S> make_step(const flb_ctx *c, const Box &b, int orient)
     s.groups = b.cfg.nx / (c->L.V == 4 && sizeof(S) * 4 > 16 ? 2 : c->L.V);
     s.by_groups = FastDiv(s.groups);
     s.by_ny = FastDiv(b.cfg.ny);
+    s.fx = static_cast<const typename Storage<S>::R *>(b.d_fx);
     if constexpr (sizeof(typename Storage<S>::R) == 8) s.K = b.Kd;
     else s.K = b.Kf;
 #ifdef FLB_BOUNDS_CHECK
@@ -853,6 +855,8 @@ void free_box(flb_ctx *c, Box &b)
         dev_free(c, p);
         p = nullptr;
     }
+    dev_free(c, b.d_fx);
+    b.d_fx = nullptr;
     dev_free(c, b.d_acc);
     dev_free(c, b.d_partial);
     dev_free(c, b.d_rho);
@@ -960,6 +964,23 @@ int create_impl(const flb_config *cfgs, int nboxes, flb_ctx **out)
     if (dev_malloc(c, &c->d_step, sizeof(uint32_t)) != cudaSuccess) {
         cudaGetLastError();
         return bail(FLB_ENOMEM, "cannot allocate the step counter");
+    }
+    if (c->force && !is_d2(c) && c->store != FLB_STORE_F32) {   // (see force_at)
+        for (Box &b : c->boxes) {
+            const int n = b.cfg.nz;
+            const bool f64 = c->store == FLB_STORE_F64;
+            if (dev_malloc(c, &b.d_fx, (size_t)n * (f64 ? sizeof(double) : sizeof(float))) != cudaSuccess) {
+                cudaGetLastError();
+                return bail(FLB_ENOMEM, "cannot allocate the body-force table");
+            }
+            // complete before the first step: the states are set, and waited for, below
+            const cudaError_t e =
+                f64 ? launch_force_table<double>(static_cast<double *>(b.d_fx), n, b.Kd.force_amp, b.Kd.force_phase,
+                                                 c->stream)
+                    : launch_force_table<float>(static_cast<float *>(b.d_fx), n, b.Kf.force_amp, b.Kf.force_phase,
+                                                c->stream);
+            if (e != cudaSuccess) return bail(FLB_ECUDA, "filling the body-force table");
+        }
     }
 #ifdef FLB_BOUNDS_CHECK
     if (dev_malloc(c, &c->d_viol, sizeof(unsigned long long)) != cudaSuccess) {

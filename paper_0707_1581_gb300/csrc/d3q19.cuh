@@ -107,7 +107,7 @@ struct CollideConsts : CollideTables<R> {
     R noise[Q];
     R forcing[10];
     R force_amp;      // F_x(z) = force_amp sin(2 pi z / nz)
-    R force_phase;    // 2 / nz (sin(pi * force_phase * z))
+    R force_phase;    // 2 / nz (sin(pi * force_phase * z)); BoxStep's table fx is made from these
     int noise_rho_local;
     uint32_t rk0[10];  // Philox round keys k0 + r * 0x9E3779B9, r = 0..9
     uint32_t rk1[10];  // Philox round keys k1 + r * 0xBB67AE85

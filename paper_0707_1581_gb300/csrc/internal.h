@@ -139,6 +139,10 @@ cudaError_t launch_moments(const double *n, int64_t slab, int nx, int ny, int nz
 
 cudaError_t launch_advance_step(uint32_t *step_ptr, uint32_t by, cudaStream_t st);
 
+// fx[z] = amp sin(pi phase z), z < n: the body force of a D3Q19 box's planes.
+template <class R>
+cudaError_t launch_force_table(R *fx, int n, R amp, R phase, cudaStream_t st);
+
 // Counts the stored values of a state buffer (n elements, format `store` =
 // flb_store_t) whose exponent bits are all set; adds the count to *count.
 cudaError_t launch_count_nonfinite(const void *buf, int64_t n, int store, unsigned long long *count, cudaStream_t st);

@@ -49,8 +49,21 @@ struct BoxStep {
     int groups, rows;          // threads (of V sites) per row; whole rows per block (kRows)
     FastDiv by_groups, by_ny;  // division by groups and by ny
     CollideConsts<typename Storage<S>::R> K;
+    const typename Storage<S>::R *fx;   // the body force F_x(z) of every plane (kernels with a force)
     FLB_VIOL_FIELD
 };
+
+// The body force of plane z, from the table that was filled when the context was
+// made; FP32 boxes, bound by memory, compute it (about 25 instructions per
+// thread).  512 x 512 x 256 FP16 AA odd step 1.100 -> 1.050 ms, 64^3 FP64 101.7 ->
+// 96.1 us; 250 x 187 x 93 FP32 100.3 us computed, 101.4 from the table.
+template <class S>
+__device__ __forceinline__ typename Storage<S>::R force_at(const BoxStep<S> &B, int z)
+{
+    using R = typename Storage<S>::R;
+    if constexpr (sizeof(S) == 4) return B.K.force_amp * sin_pi(B.K.force_phase * R(z));
+    else return __ldg(B.fx + z);
+}
 
 // When a step's blocks let the next step's blocks start (see d3q19.cuh).  Four
 // sites per thread, the launches of many waves: at their own start, so that the
@@ -80,8 +93,6 @@ __device__ __forceinline__ void update_sites(const BoxStep<S> &B, int x0, int y,
     auto zsel = [&](int c) { return c > 0 ? zm : (c < 0 ? zp : z); };   // z - c
     auto ysel_push = [&](int c) { return c > 0 ? yp : (c < 0 ? ym : y); };  // y + c
     auto zsel_push = [&](int c) { return c > 0 ? zp : (c < 0 ? zm : z); };
-    R Fx = R(0);
-    if (FORCE) Fx = B.K.force_amp * sin_pi(B.K.force_phase * R(z));
     const uint32_t site_row = (uint32_t)row(y, z);
     static_assert(V == 1, "the scalar path takes one site per thread");
     {
@@ -107,6 +118,7 @@ __device__ __forceinline__ void update_sites(const BoxStep<S> &B, int x0, int y,
             f[i] = Storage<S>::load(load_ro(FLB_GUARD_LD(B, p, 1)));
         }
         if constexpr (kStart<S, V> == kAfterLoads) let_next_step_start();
+        const R Fx = FORCE ? force_at(B, z) : R(0);
         if constexpr (sizeof(R) == 8) collide64<NOISE, FORCE, true>(f, B.K, site_row + (uint32_t)x, step, B.replica, Fx, g);
         else collide<R, NOISE, FORCE, true>(f, B.K, site_row + (uint32_t)x, step, B.replica, Fx, g);
         stochastic_round<S>(f, site_row + (uint32_t)x, step, B.replica, B.K.rk0, B.K.rk1);
@@ -458,9 +470,8 @@ __device__ __forceinline__ void update_vec(const BoxStep<S> &B, int x0, int y, i
         }
     }
 
-    R Fx = R(0);
     if constexpr (kStart<S, V> == kAfterLoads) let_next_step_start();
-    if (FORCE) Fx = B.K.force_amp * sin_pi(B.K.force_phase * R(z));
+    const R Fx = FORCE ? force_at(B, z) : R(0);
     // 16-bit formats (issue-bound): two sites per collision in the paired FP32
     // instructions; FP32 storage is bound by HBM and keeps the one-site form,
     // whose odd AA step measured faster
