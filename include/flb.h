@@ -113,7 +113,8 @@ typedef struct {
     int sites_per_thread;      /* 0 = automatic (4, FP64 2; halved while the boxes' sites
                                   over it stay below 100,000 threads); else 1, 2 or 4
                                   (x-consecutive sites) */
-    int block_x, block_y;      /* 0 = automatic; else the CUDA block shape */
+    int block_x, block_y;      /* 0 = automatic; else the threads of a block, block_x * block_y (how a D3Q19
+                                  block covers the box's rows follows from them and nx) */
     int graph_steps;           /* steps per captured CUDA graph; 0 = plain launches */
     int lattice;               /* flb_lattice_t; every box of a context has the same lattice */
     int stats_every;           /* k > 0: flb_step takes a statistics sample (flb_stats_sample) after
@@ -175,9 +176,10 @@ int flb_step(flb_ctx *ctx, int64_t nsteps);
  * of flb_box_state_download, flb_box_state_bytes long; pinned memory for full
  * speed).  The call uploads it, advances the context by nsteps (Eq. LBE with
  * the collision of Sec. IV) and writes the new state back to `host`.  The
- * first step runs in z-chunks as the planes arrive, on a copy stream beside the
- * compute stream, and the downloads start chunk by chunk as the step finishes
- * them, so the two copy directions and the kernel overlap.  Other boxes of a
+ * first step (of a single box: the first few, each some chunks behind the one
+ * before) runs in z-chunks as the planes arrive, on a copy stream beside the
+ * compute stream, and the downloads start chunk by chunk as the last of them
+ * finishes, so the two copy directions and the kernels overlap.  Other boxes of a
  * batch do not advance their state, but the step counter is shared.  D3Q19 only
  * (FLB_EINVAL for D2Q9).  Synchronises. */
 int flb_box_step_host(flb_ctx *ctx, int box, void *host, int64_t nsteps);

@@ -139,3 +139,28 @@ def test_host_resident_steps_in_a_wave_equal_device_steps(pattern, start, nz, ns
         assert np.array_equal(raw(ctx), want)
         ctx.flb_step(3)
         assert np.array_equal(raw(ctx), later)
+
+
+@pytest.mark.parametrize("nx,store,kw", [(16, "f32", {}), (64, "f16dev", {}), (128, "f32", {}), (16, "f64", {}),
+                                         (64, "f32", dict(lattice="d2q9"))])
+def test_chained_launches_in_a_callers_graph(nx, store, kw):
+    """Steps and a statistics sample captured from the caller's stream do what they do outside a capture."""
+    import torch
+
+    stream = torch.cuda.Stream()
+    ny, nz = (nx, 1) if kw else (nx, nx // 2)
+    with flb.flb_create_ex(box(nx, ny, nz, store, "ab", **kw)) as ctx:
+        ctx.flb_step(4)
+        ctx.flb_stats_sample()
+        want, stats = raw(ctx), ctx.flb_mode_stats()
+    with flb.flb_create_ex(box(nx, ny, nz, store, "ab", stream=stream, **kw)) as ctx:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            ctx.flb_step(4)
+            ctx.flb_stats_sample()
+        with torch.cuda.stream(stream):
+            graph.replay()
+        assert np.array_equal(raw(ctx), want)
+        got = ctx.flb_mode_stats()
+        assert got["nsamples"] == 1 and np.array_equal(got["mode_m2"], stats["mode_m2"])
+        del graph
