@@ -1222,9 +1222,14 @@ int flb_box_step_host(flb_ctx *c, int box, void *host, int64_t nsteps)
     // step before is done on that chunk and on both beside it, so the downloads
     // start a few chunks behind the uploads and both copy directions run together
     // (256^3 FP32, two steps: 8.5 ms, 13.2 with the downloads behind the last
-    // step).  More steps than an eighth of the chunks, and batches, whose other
-    // boxes take part in the further steps, step whole boxes.
-    const bool wave = nsteps > 1 && K >= 8 && nsteps - 1 <= K / 8 && c->boxes.size() == 1;
+    // step).  A further step in chunks is K launches, about 0.1 ms of the host, and
+    // the wave saves at most the time of one copy of the state, so it wants 20 MB of
+    // state for each (two steps: 12 MB 1.03x, 32 MB 1.19x; four: 21 MB 0.73x, 42 MB
+    // 0.95x, 66 MB 1.21x).  Smaller states, more steps than an eighth of the chunks,
+    // and batches, whose other boxes take part in the further steps, step whole boxes.
+    constexpr int64_t kWaveBytes = 20000000;
+    const bool wave = nsteps > 1 && K >= 8 && nsteps - 1 <= K / 8 && c->boxes.size() == 1 &&
+                      state_bytes >= (nsteps - 1) * kWaveBytes;
     const int nwave = wave ? (int)nsteps : 1;
     for (int tau = 0; tau < K + 2 * (nwave - 1); ++tau) {
         for (int s = 0; s < nwave; ++s) {

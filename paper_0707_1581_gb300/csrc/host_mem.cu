@@ -68,14 +68,16 @@ void prefault(void *p, size_t bytes)
     // whole pages inside the array
     const uintptr_t a = ((uintptr_t)p + page - 1) / page * page, b = ((uintptr_t)p + bytes) / page * page;
     if (b <= a) return;
-    // nothing to do when a spread of its pages is there (asking anyway takes 1.5 ms for 319 MB)
-    bool resident = true;
-    for (int k = 0; k < 32 && resident; ++k) {
-        unsigned char in = 0;
-        const uintptr_t at = a + ((b - a) / page - 1) * k / 31 * page;
-        resident = mincore((void *)at, page, &in) == 0 && (in & 1);
+    // nothing to do when its pages are there: one look at all of them (a call per page
+    // looked at took 0.5 us each, 18 us of the 160 that a 24^3 box's fields take;
+    // populating them anyway 1.5 ms for 319 MB)
+    try {
+        std::vector<unsigned char> in((b - a) / page);
+        if (mincore((void *)a, b - a, in.data()) == 0 &&
+            std::all_of(in.begin(), in.end(), [](unsigned char x) { return x & 1; }))
+            return;
+    } catch (...) {   // no memory for the look
     }
-    if (resident) return;
     const size_t n = std::max<size_t>(1, std::min<size_t>({8, (b - a) / kPerThread, std::thread::hardware_concurrency()}));
     const uintptr_t step = ((b - a) / n + page - 1) / page * page;
     auto part = [=](size_t k) {

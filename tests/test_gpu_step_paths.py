@@ -119,11 +119,13 @@ def test_automatic_launch_fits_its_box_and_is_accepted_back(nx, store):
         assert np.array_equal(raw(ctx), want)
 
 
-@pytest.mark.parametrize("nz,nsteps", [(8, 2), (9, 2), (31, 4), (32, 5), (40, 5), (40, 6), (7, 3)])
+@pytest.mark.parametrize("nx,ny,nz,nsteps", [(256, 130, 8, 2), (256, 117, 9, 2), (256, 100, 31, 4), (256, 129, 32, 5),
+                                             (256, 104, 40, 5)] +
+                         [(24, 6, nz, n) for nz, n in [(8, 2), (9, 2), (31, 4), (32, 5), (40, 5), (40, 6), (7, 3)]])
 @pytest.mark.parametrize("pattern,start", [("ab", 0), ("ab", 1), ("aa", 0), ("aa", 1)])
-def test_host_resident_steps_in_a_wave_equal_device_steps(pattern, start, nz, nsteps):
-    """Several steps per call, each a few chunks behind the one before (7 chunks and 6 steps of 32: whole boxes)."""
-    cfg = box(24, 6, nz, "f32", pattern, kT=1e-3, force_amp=1e-4)
+def test_host_resident_steps_in_a_wave_equal_device_steps(pattern, start, nx, ny, nz, nsteps):
+    """Several steps per call, each a few chunks behind the one before (20 MB of state for each; less: whole boxes)."""
+    cfg = box(nx, ny, nz, "f32", pattern, kT=1e-3, force_amp=1e-4)
     with flb.flb_create_ex(cfg) as ref:
         ref.flb_step(6 + start)
         host = raw(ref)
