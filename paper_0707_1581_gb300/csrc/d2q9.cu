@@ -32,15 +32,64 @@ constexpr int vec_width()
     return sizeof(S) == 8 ? 2 : 4;
 }
 
+// When a step's blocks let the next step's blocks start.  Any sooner than the SMs
+// have room for them without waiting, and they crowd onto the SMs that happen to
+// be free, which unbalances every later step; so boxes of about a block per SM
+// wait for their loads, and 16-bit boxes of two for their stores.  Beyond that
+// 16-bit formats, bound by instructions, start at once, and FP32 waits for its
+// stores while the state lies in L2 and for its loads when it streams from HBM
+// (the compiler also keeps every load ahead of that point).  us per step, AB,
+// unchained / at the start / after the loads / before the stores:
+//   FP16  236 x 551 (128 blocks)  4.17 / 4.85 / 2.90 / 2.68; AA in graphs 3.33 / 4.14 / 3.14 / 3.56
+//         512 x 512 (256)         6.20 / 5.03 / 4.99 / 3.81
+//         1024^2 (1024)           12.35 / 10.12 / 10.18 / 10.16;  3000 x 2400  65.2 / 62.8 / 65.9 / 63.0
+//   FP32  236 x 551               6.19 / 6.27 / 3.45 / 3.53
+//         752 x 437 (321)         8.24 / 7.37 / 6.39 / 5.47
+//         1744 x 864 (1472)       18.49 / 16.08 / 17.10 / 16.24;  3000 x 2400  86.9 / 86.2 / 78.1 / 84.9
+template <class S, int LAYOUT>
+StartPoint start_point(const BoxStep<S> &b, int64_t blocks, bool in_graph)   // of 256 threads
+{
+    constexpr int64_t kSMs = 152;
+    constexpr int64_t kL2 = 128000000;
+    if (sizeof(S) == 8) return kAfterLoads;
+    if (sizeof(S) == 2) return blocks <= kSMs ? kAfterLoads : blocks <= 2 * kSMs ? kBeforeStores : kAtStart;
+    const bool in_l2 = (LAYOUT == kAB ? 2 : 1) * Q * b.plane * (int64_t)sizeof(S) <= kL2;
+    // a graph's launches are close enough for a state in L2: 632 x 640 FP32 takes 5.82 us
+    // unchained and 6.93 / 6.22 chained, the boxes of 25,600 to 1.5 M sites at most 3 % less
+    if (in_l2 && in_graph) return kUnchained;
+    return in_l2 && blocks > 2 * kSMs ? kBeforeStores : kAfterLoads;
+}
+
+template <class S, int LAYOUT, bool NOISE, bool FORCE>
+cudaError_t step_vec(const BoxStep<S> &b, dim3 grid, dim3 block, const uint32_t *p, uint32_t t, cudaStream_t st)
+{
+    constexpr int V = vec_width<S>();
+    const StartPoint at = start_point<S, LAYOUT>(b, (int64_t)grid.x * block.x * block.y / 256, p != nullptr);
+    if constexpr (sizeof(S) == 2) {
+        if (at == kAtStart)
+            return launch_chained(k_stream_collide_vec<S, LAYOUT, NOISE, FORCE, V, kAtStart>, grid, block, st, b, p, t);
+    }
+    if constexpr (sizeof(S) < 8) {
+        if (at == kBeforeStores)
+            return launch_chained(k_stream_collide_vec<S, LAYOUT, NOISE, FORCE, V, kBeforeStores>, grid, block, st, b, p, t);
+    }
+    if constexpr (sizeof(S) == 4) {
+        if (at == kUnchained) {
+            k_stream_collide_vec<S, LAYOUT, NOISE, FORCE, V, kBeforeStores><<<grid, block, 0, st>>>(b, p, t);
+            return cudaGetLastError();
+        }
+    }
+    return launch_chained(k_stream_collide_vec<S, LAYOUT, NOISE, FORCE, V, kAfterLoads>, grid, block, st, b, p, t);
+}
+
 template <class S, int LAYOUT>
 cudaError_t step_layout_vec(const BoxStep<S> &b, bool noise, bool force, dim3 grid, dim3 block, const uint32_t *p,
                             uint32_t t, cudaStream_t st)
 {
-    constexpr int V = vec_width<S>();
-    if (noise && force) return launch_chained(k_stream_collide_vec<S, LAYOUT, true, true, V>, grid, block, st, b, p, t);
-    if (noise) return launch_chained(k_stream_collide_vec<S, LAYOUT, true, false, V>, grid, block, st, b, p, t);
-    if (force) return launch_chained(k_stream_collide_vec<S, LAYOUT, false, true, V>, grid, block, st, b, p, t);
-    return launch_chained(k_stream_collide_vec<S, LAYOUT, false, false, V>, grid, block, st, b, p, t);
+    if (noise && force) return step_vec<S, LAYOUT, true, true>(b, grid, block, p, t, st);
+    if (noise) return step_vec<S, LAYOUT, true, false>(b, grid, block, p, t, st);
+    if (force) return step_vec<S, LAYOUT, false, true>(b, grid, block, p, t, st);
+    return step_vec<S, LAYOUT, false, false>(b, grid, block, p, t, st);
 }
 
 }  // namespace

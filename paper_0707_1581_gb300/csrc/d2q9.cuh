@@ -274,17 +274,13 @@ __device__ __forceinline__ void store_vec2(S *p, const S (&in)[V])
     *reinterpret_cast<T *>(p) = raw;
 }
 
-template <class S, int LAYOUT, bool NOISE, bool FORCE, int V>
+// START: when a step's blocks let the next step's start (start_point in d2q9.cu has the rule)
+template <class S, int LAYOUT, bool NOISE, bool FORCE, int V, int START>
 __global__ void __launch_bounds__(256, sizeof(typename Storage<S>::R) == 4 ? (sizeof(S) == 2 ? 3 : 4) : 1)
 k_stream_collide_vec(const BoxStep<S> B, const uint32_t *step_ptr, uint32_t step)
 {
     using R = typename Storage<S>::R;
-    // The next step may start behind this one's loads (32-bit formats: the 8192^2
-    // FP32 AB step takes 693 us so, 742 with it let in at the start, 718 unchained;
-    // the compiler also keeps every load ahead of that point), or at the start
-    // (16-bit formats: 521 us FP16 AB, 554 behind the loads)
-    constexpr bool kAtStart = sizeof(S) == 2;
-    if constexpr (kAtStart) let_next_step_start();
+    if constexpr (START == kAtStart) let_next_step_start();
     const int nx = B.nx, ny = B.ny, gx = nx / V;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int lane = tid & 31;
@@ -314,7 +310,7 @@ k_stream_collide_vec(const BoxStep<S> B, const uint32_t *step_ptr, uint32_t step
         if (LAYOUT != kAAEven && cx > 0) edge[i] = load_ro(FLB_GUARD_LD(B, base + x_lload, 1));
         if (LAYOUT != kAAEven && cx < 0) edge[i] = load_ro(FLB_GUARD_LD(B, base + x_rload, 1));
     }
-    if constexpr (!kAtStart) let_next_step_start();
+    if constexpr (START == kAfterLoads) let_next_step_start();
     R f[V][Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -358,6 +354,7 @@ k_stream_collide_vec(const BoxStep<S> B, const uint32_t *step_ptr, uint32_t step
     }
 #pragma unroll
     for (int v = 0; v < V; ++v) stochastic_round<S>(f[v], site0 + v, step, B.replica, B.K.rk0, B.K.rk1);
+    if constexpr (START == kBeforeStores) let_next_step_start();
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const int cx = vel_x(i), cy = vel_y(i);

@@ -783,6 +783,10 @@ __device__ __forceinline__ bool span_ok(const S *base, int64_t plane, const S *p
 __device__ __forceinline__ void let_next_step_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous_step() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Where a step kernel calls let_next_step_start (kUnchained: launched without
+// programmatic serialization, where that is the faster).
+enum StartPoint : int { kUnchained = -1, kAtStart = 0, kAfterLoads = 1, kBeforeStores = 2 };
+
 // --------------------------------------------------------------------------
 // Where the canonical pre-collision population n_i(r, t) lives in device memory.
 //   AB (pull):     slot i at r - c_i of the current buffer (it holds the

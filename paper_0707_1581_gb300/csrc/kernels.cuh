@@ -76,7 +76,6 @@ __device__ __forceinline__ typename Storage<S>::R force_at(const BoxStep<S> &B, 
 // unchained launches): 64^3 FP32 6.26 / 6.02 / 5.94 us, 48^3 FP32 5.32 / 3.80 /
 // 4.03, 16^3 FP32 2.26 / 1.69 / 1.92, 16^3 FP64 8.26 / 8.06 / 7.84, 32^3 FP64
 // 39.9 / 16.6 / 16.1; V = 4: 96^3 FP32 28.8 / 29.8 / 29.1.
-enum StartPoint : int { kAtStart = 0, kAfterLoads = 1, kBeforeStores = 2 };
 template <class S, int V>
 constexpr StartPoint kStart = sizeof(S) == 8 ? kBeforeStores : (V >= 4 ? kAtStart : kAfterLoads);
 

@@ -166,3 +166,19 @@ def test_chained_launches_in_a_callers_graph(nx, store, kw):
         got = ctx.flb_mode_stats()
         assert got["nsamples"] == 1 and np.array_equal(got["mode_m2"], stats["mode_m2"])
         del graph
+
+
+@pytest.mark.parametrize("nx,ny", [(236, 551), (512, 512), (752, 437), (1024, 1024), (2048, 2100)])
+@pytest.mark.parametrize("store", ["f64", "f32", "f16dev", "bf16sr"])
+@pytest.mark.parametrize("pattern,graph_steps", [("ab", 0), ("aa", 0), ("ab", 10), ("aa", 10)])
+def test_chained_d2q9_steps_equal_steps_one_at_a_time(pattern, graph_steps, store, nx, ny):
+    """Boxes of one block per SM, two, more, and beyond L2: each start point of the next step."""
+    cfg = dict(lattice="d2q9", kT=1e-4, force_amp=1e-5)
+    with flb.flb_create_ex(box(nx, ny, 1, store, pattern, **cfg)) as ctx:
+        for _ in range(21):
+            ctx.flb_step(1)
+            ctx.flb_sync()
+        want = raw(ctx)
+    with flb.flb_create_ex(box(nx, ny, 1, store, pattern, graph_steps=graph_steps, **cfg)) as ctx:
+        ctx.flb_step(21)
+        assert np.array_equal(raw(ctx), want)
