@@ -127,6 +127,13 @@ __global__ void __launch_bounds__(kThreads) k_unit_sums(const S *__restrict__ bu
     if (tid == 0) part[((int64_t)q * units + u) * chunks + c] = sum;
 }
 
+// The unit of a thread of k_unit_means.  Warps are counted, not threads: 2^27 units have
+// 2^32 threads.
+__host__ __device__ inline int unit_of(unsigned block, unsigned block_threads, unsigned thread)
+{
+    return (int)(block * (block_threads / 32) + thread / 32);
+}
+
 // Warp u: out[u] = rho0 + sum_i s_i / M, out[units + 3 u + a] = sum_i c_ia s_i / M,
 // s_i (lane i) the sum of the deviation n_i over unit u.  D2: the D2Q9 velocities
 // in rows y (the third component is 0).
@@ -135,7 +142,7 @@ __global__ void __launch_bounds__(128) k_unit_means(const double *__restrict__ p
                                                     int chunks, double rho0, double *__restrict__ out)
 {
     constexpr int NQ = D2 ? 9 : 19;
-    const int i = (int)threadIdx.x & 31, u = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int i = (int)threadIdx.x & 31, u = unit_of(blockIdx.x, blockDim.x, threadIdx.x);
     if (u >= units) return;   // whole warps
     constexpr int vx[2][19] = {{0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1},
                                {0, 1, -1, 0, 0, 1, -1, 1, -1}};

@@ -69,3 +69,20 @@ def test_profile_of_values_beyond_the_ordinary(store):
                 want_rho, want_j = reference(ctx.flb_get_populations(), False)
             assert np.array_equal(np.isnan(rho), np.isnan(want_rho)) and np.array_equal(np.isinf(rho), np.isinf(want_rho))
             assert np.array_equal(np.isnan(j), np.isnan(want_j)) and np.array_equal(np.isinf(j), np.isinf(want_j))
+
+
+def test_profile_of_more_than_2_to_27_rows():
+    """D2Q9 rows of four sites; one thermal step, rows around 2^27 and the ends against their populations."""
+    torch = pytest.importorskip("torch")
+    ny = 2 ** 27 + 100                      # 2^29 sites, 9.7 GB of bfloat16 state
+    if torch.cuda.mem_get_info()[0] < 24e9:
+        pytest.skip("needs 24 GB of free device memory")
+    rows = np.array([0, 1, 99, 100, 2 ** 26, 2 ** 27 - 1, 2 ** 27, 2 ** 27 + 1, ny - 2, ny - 1])
+    cfg = flb.config(4, ny, 1, kT=1e-3, gamma_shear=0.3, seed=2, store="bf16dev", pattern="aa", lattice="d2q9")
+    with flb.flb_create_ex(cfg) as ctx:
+        ctx.flb_step(1)
+        n = ctx.flb_get_sites((4 * rows[:, None] + np.arange(4)).ravel()).reshape(len(rows), 4, 9)
+        rho, j = ctx.flb_z_profile()
+    want_rho, want_j = reference(n.transpose(2, 0, 1), True)
+    # as in the test above
+    assert np.abs(rho[rows] - want_rho).max() <= 2e-14 and np.abs(j[:, rows] - want_j).max() <= 2e-14
