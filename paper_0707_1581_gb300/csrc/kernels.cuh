@@ -315,14 +315,15 @@ struct RowExchange {
 
 // A thread's place in its block's rows (kOneRow, kRows): which ends it owns,
 // and the exchange slots that it writes (mine_*) and reads (from_*).  A row end
-// has the row's slot; a warp end inside a row has the warp's.
+// has the row's slot; a warp end inside a row has the warp's.  A thread beyond the
+// block's rows gets slots inside the arrays too; what it reads there is not used.
 struct RowPlace {
     bool give_last, give_first;    // the right (left) neighbour cannot reach this thread by shuffle
     bool take_left, take_right;    // the left (right) neighbour's element comes from the exchange
     int mine_last, mine_first, from_left, from_right;
 };
 template <int XCH>
-__device__ __forceinline__ RowPlace row_place(int lane, int warp, int nwarp, int tx, int g, int row)
+__host__ __device__ __forceinline__ RowPlace row_place(int lane, int warp, int nwarp, int tx, int g, int row)
 {
     RowPlace p;
     if constexpr (XCH == kOneRow) {
@@ -339,7 +340,8 @@ __device__ __forceinline__ RowPlace row_place(int lane, int warp, int nwarp, int
         p.mine_last = end ? row : kRowSlots + warp;
         p.mine_first = start ? row : kRowSlots + warp;
         p.from_left = start ? row : kRowSlots + (lane == 0 ? warp - 1 : warp);
-        p.from_right = end ? row : kRowSlots + (lane == 31 ? warp + 1 : warp);
+        const int next = warp + 1 < kXchWarps ? warp + 1 : warp;   // the last warp's last lane ends a row, or is idle
+        p.from_right = end ? row : kRowSlots + (lane == 31 ? next : warp);
     }
     return p;
 }

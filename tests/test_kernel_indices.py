@@ -32,3 +32,42 @@ def test_every_unit_has_its_own_warp_of_the_plane_means(tmp_path, units):
                 return 1;
             }}
         }}""", "profile.cuh")
+
+
+@pytest.mark.parametrize("xch", ["kRows", "kRagRow", "kOneRow"])
+def test_row_exchange_slots_lie_in_the_arrays_and_pair_up(tmp_path, xch):
+    """Every thread of every block shape that the exchange can have, the idle ones among them: slots inside the
+    arrays; a thread with a site group reads what its neighbour in the (periodic) row wrote."""
+    run_host(tmp_path, f"""
+    constexpr int X = {xch}, slots = RowExchange<float, X>::kSlots;
+    int bad = 0;
+    for (int g = 1; g <= 256; ++g)
+        for (int rows = 1; rows <= kXchRows && rows * g <= 256; ++rows)
+            for (int T = (rows * g + 31) / 32 * 32; T <= 256; T += 32) {{
+                if (X != kRows && rows > 1) continue;
+                if (X == kOneRow && T != g) continue;
+                auto place = [&](int t) {{
+                    const int tr = t / g, tx = X == kRows ? t - tr * g : (t < g ? t : g - 1);
+                    return row_place<X>(t & 31, t >> 5, T / 32, tx, g, X == kRows ? (tr < kXchRows ? tr : kXchRows - 1) : 0);
+                }};
+                int last[slots], first[slots];
+                for (int k = 0; k < slots; ++k) last[k] = first[k] = -1;
+                for (int t = 0; t < T; ++t) {{
+                    const RowPlace p = place(t);
+                    for (int k : {{p.mine_last, p.mine_first, p.from_left, p.from_right}})
+                        if (k < 0 || k >= slots) {{
+                            if (!bad++) printf("g %d rows %d T %d thread %d: slot %d of %d\\n", g, rows, T, t, k, slots);
+                        }}
+                    if (t >= rows * g) continue;
+                    if (p.give_last) last[p.mine_last] = last[p.mine_last] < 0 ? t : -2;      // -2: two writers
+                    if (p.give_first) first[p.mine_first] = first[p.mine_first] < 0 ? t : -2;
+                }}
+                for (int t = 0; t < rows * g; ++t) {{
+                    const RowPlace p = place(t);
+                    const int r = t / g, x = t - r * g, left = r * g + (x + g - 1) % g, right = r * g + (x + 1) % g;
+                    if (p.take_left ? last[p.from_left] != left : left != t - 1) ++bad;
+                    if (p.take_right ? first[p.from_right] != right : right != t + 1) ++bad;
+                }}
+            }}
+    if (bad) printf("%d\\n", bad);
+    return bad != 0;""", "kernels.cuh")
