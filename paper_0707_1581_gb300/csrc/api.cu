@@ -1008,7 +1008,7 @@ int create_impl(const flb_config *cfgs, int nboxes, flb_ctx **out)
     return FLB_OK;
 }
 
-cudaError_t profile_box(flb_ctx *c, const Box &b, double *part, double *out)
+cudaError_t profile_box(flb_ctx *c, const Box &b, const profile::Pass &P, double *part, double *out)
 {
     const bool two = is_d2(c);
     const int layout = layout_of(c, c->step), n = units(b);
@@ -1016,16 +1016,16 @@ cudaError_t profile_box(flb_ctx *c, const Box &b, double *part, double *out)
     const void *buf = state_buf(c, b);
     switch (c->store) {
     case FLB_STORE_F64:
-        return launch_profile<double>(static_cast<const double *>(buf), b.plane, layout, M, n, two, b.cfg.rho0, part, out,
+        return launch_profile<double>(static_cast<const double *>(buf), b.plane, layout, M, n, P, two, b.cfg.rho0, part, out,
                                       c->stream);
     case FLB_STORE_F32:
-        return launch_profile<float>(static_cast<const float *>(buf), b.plane, layout, M, n, two, b.cfg.rho0, part, out,
+        return launch_profile<float>(static_cast<const float *>(buf), b.plane, layout, M, n, P, two, b.cfg.rho0, part, out,
                                      c->stream);
     case FLB_STORE_F16DEV:
-        return launch_profile<__half>(static_cast<const __half *>(buf), b.plane, layout, M, n, two, b.cfg.rho0, part, out,
+        return launch_profile<__half>(static_cast<const __half *>(buf), b.plane, layout, M, n, P, two, b.cfg.rho0, part, out,
                                       c->stream);
     default:   // both bfloat16 formats hold the same bits
-        return launch_profile<__nv_bfloat16>(static_cast<const __nv_bfloat16 *>(buf), b.plane, layout, M, n, two,
+        return launch_profile<__nv_bfloat16>(static_cast<const __nv_bfloat16 *>(buf), b.plane, layout, M, n, P, two,
                                              b.cfg.rho0, part, out, c->stream);
     }
 }
@@ -1430,28 +1430,33 @@ int flb_box_z_profile(flb_ctx *c, int box, double *rho, double *j)
     Box *b = box_of(c, box);
     if (!b) return fail(c, FLB_EINVAL, "bad box index");
     const int nz = units(*b);            // z-planes, or y-rows of a D2Q9 box
-    const size_t part = (size_t)b->Q * nz * profile_chunks(unit_sites(*b), nz, b->Q), means = 4 * (size_t)nz;
+    const profile::Pass most = profile::pass_from(0, nz);
+    const size_t part = (size_t)b->Q * most.nsum * profile_chunks(unit_sites(*b), nz, b->Q), means = 4 * (size_t)most.n;
     int rc = ensure_scratch(c, (part + means) * sizeof(double));
     if (rc) return rc;
     // the means are written straight to page-locked memory where there is some
     std::vector<double> own;
     double *h = static_cast<double *>(result_memory(c, means * sizeof(double)));
     double *out = h ? h : c->d_scratch + part;
-    CK(c, profile_box(c, *b, c->d_scratch, out));
-    if (!h) {
-        own.resize(means);
-        h = own.data();
-        CK(c, cudaMemcpyAsync(h, out, means * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    }
-    CK(c, cudaStreamSynchronize(c->stream));
-    for (int z = 0; z < nz; ++z) {
-        if (rho) rho[z] = h[z];
-        if (j) {
-            // half-step momentum with a body force (see flb_box_moments)
-            const double half_force = 0.5 * b->cfg.force_amp * std::sin(2.0 * M_PI * z / nz);
-            j[z] = h[nz + 3 * z] + half_force;
-            j[nz + z] = h[nz + 3 * z + 1];
-            j[2 * nz + z] = h[nz + 3 * z + 2];
+    if (!h) own.resize(means);
+    for (int64_t u0 = 0; u0 < nz; u0 += most.n) {
+        const profile::Pass P = profile::pass_from((int)u0, nz);
+        CK(c, profile_box(c, *b, P, c->d_scratch, out));
+        if (!own.empty()) {
+            h = own.data();
+            CK(c, cudaMemcpyAsync(h, out, 4 * (size_t)P.n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        }
+        CK(c, cudaStreamSynchronize(c->stream));
+        for (int k = 0; k < P.n; ++k) {
+            const int64_t z = u0 + k;
+            if (rho) rho[z] = h[k];
+            if (j) {
+                // half-step momentum with a body force (see flb_box_moments)
+                const double half_force = 0.5 * b->cfg.force_amp * std::sin(2.0 * M_PI * z / nz);
+                j[z] = h[P.n + 3 * k] + half_force;
+                j[nz + z] = h[P.n + 3 * k + 1];
+                j[2 * (int64_t)nz + z] = h[P.n + 3 * k + 2];
+            }
         }
     }
     return FLB_OK;

@@ -48,24 +48,52 @@ struct PairSum {
 constexpr int kThreads = 256;     // per block
 constexpr int kUnroll = 4;        // 16-byte loads in flight per thread
 
-// T threads (a warp or the block) sum chunk c of `chunks` of unit u of slot q, M
-// elements per unit, into part[(q units + u) chunks + c]; work item w is (c, q, u)
-// with u fastest.
+// The units of one pass: the sums of nsum consecutive units from `first` on (modulo
+// the box's units), then the means of n units, of which the first is the lead-th
+// sum.  A box of at most kPassUnits units is one pass over all of its sums (lead =
+// 0, the neighbours of the ends wrap around); a larger one takes kPassUnits at a
+// time with one sum more at either side (lead = 1), so that the scratch stays at
+// 4 units + Q nsum doubles (10 MB) and the indices of sums and means within 32 bits.
+struct Pass {
+    int first, nsum, lead, n;
+};
+constexpr int kPassUnits = 65536;
+__host__ __device__ inline Pass pass_from(int u0, int units)
+{
+    if (units <= kPassUnits) return Pass{0, units, 0, units};
+    const int n = units - u0 < kPassUnits ? units - u0 : kPassUnits;
+    return Pass{(u0 ? u0 : units) - 1, n + 2, 1, n};
+}
+// the box's unit of sum u, and the sum that slot i's unit k of the means comes from
+__host__ __device__ inline int unit_of_sum(const Pass &p, int u, int units)
+{
+    const unsigned v = (unsigned)p.first + (unsigned)u;
+    return (int)(v < (unsigned)units ? v : v - (unsigned)units);
+}
+__host__ __device__ inline int sum_of_mean(const Pass &p, int k, int shift)
+{
+    const int u = k + p.lead - shift;
+    return u < 0 ? u + p.nsum : (u >= p.nsum ? u - p.nsum : u);
+}
+
+// T threads (a warp or the block) sum chunk c of `chunks` of sum u (unit
+// unit_of_sum) of slot q, M elements per unit, into part[(q nsum + u) chunks + c];
+// work item w is (c, q, u) with u fastest.
 template <class S, int T>
 __global__ void __launch_bounds__(kThreads) k_unit_sums(const S *__restrict__ buf, int64_t plane, int64_t M, int units,
-                                                        int64_t items, int chunks, double *__restrict__ part)
+                                                        Pass P, int64_t items, int chunks, double *__restrict__ part)
 {
     constexpr int E = 16 / sizeof(S);   // elements per 16-byte load
     constexpr int kWarps = T / 32;
     const int tid = (int)threadIdx.x % T;
     const int64_t w = (int64_t)blockIdx.x * (kThreads / T) + threadIdx.x / T;
     if (w >= items) return;             // whole warps: T is 32 or the block
-    const int u = (int)(w % units);
-    const int64_t qc = w / units;
+    const int u = (int)(w % P.nsum);
+    const int64_t qc = w / P.nsum;
     const int q = (int)(qc / chunks), c = (int)(qc % chunks);
     const int64_t per = (M + chunks - 1) / chunks, c0 = c * per;
     const int64_t n = max((int64_t)0, min(per, M - c0));
-    const S *p = buf + q * plane + u * M + c0;
+    const S *p = buf + q * plane + unit_of_sum(P, u, units) * M + c0;
     // up to the first 16-byte boundary and behind the last one: single elements
     const int64_t head = min(n, (int64_t)((16 - reinterpret_cast<uintptr_t>(p) % 16) % 16 / sizeof(S)));
     const int64_t vecs = (n - head) / E, tail = n - head - vecs * E;
@@ -124,7 +152,7 @@ __global__ void __launch_bounds__(kThreads) k_unit_sums(const S *__restrict__ bu
             for (int k = 0; k < kWarps; ++k) sum += wsum[k];
         }
     }
-    if (tid == 0) part[((int64_t)q * units + u) * chunks + c] = sum;
+    if (tid == 0) part[((int64_t)q * P.nsum + u) * chunks + c] = sum;
 }
 
 // The unit of a thread of k_unit_means.  Warps are counted, not threads: 2^27 units have
@@ -134,16 +162,16 @@ __host__ __device__ inline int unit_of(unsigned block, unsigned block_threads, u
     return (int)(block * (block_threads / 32) + thread / 32);
 }
 
-// Warp u: out[u] = rho0 + sum_i s_i / M, out[units + 3 u + a] = sum_i c_ia s_i / M,
-// s_i (lane i) the sum of the deviation n_i over unit u.  D2: the D2Q9 velocities
+// Warp u, unit u of the pass's n: out[u] = rho0 + sum_i s_i / M, out[n + 3 u + a] =
+// sum_i c_ia s_i / M, s_i (lane i) the sum of the deviation n_i over the unit.  D2: the D2Q9 velocities
 // in rows y (the third component is 0).
 template <bool D2>
-__global__ void __launch_bounds__(128) k_unit_means(const double *__restrict__ part, int layout, int64_t M, int units,
+__global__ void __launch_bounds__(128) k_unit_means(const double *__restrict__ part, int layout, int64_t M, Pass P,
                                                     int chunks, double rho0, double *__restrict__ out)
 {
     constexpr int NQ = D2 ? 9 : 19;
     const int i = (int)threadIdx.x & 31, u = unit_of(blockIdx.x, blockDim.x, threadIdx.x);
-    if (u >= units) return;   // whole warps
+    if (u >= P.n) return;   // whole warps
     constexpr int vx[2][19] = {{0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1},
                                {0, 1, -1, 0, 0, 1, -1, 1, -1}};
     constexpr int vy[2][19] = {{0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 1, -1, 1, -1, 0, 0, 0, 0},
@@ -160,8 +188,8 @@ __global__ void __launch_bounds__(128) k_unit_means(const double *__restrict__ p
     double s = 0.0;
     if (i < NQ) {
         const int q = layout == kAAOdd && i ? ((i & 1) ? i + 1 : i - 1) : i;
-        const int from = layout == kAAEven ? u : wrap_add(u, -(D2 ? cy : cz), units);
-        const double *p = part + ((int64_t)q * units + from) * chunks;
+        const int from = sum_of_mean(P, u, layout == kAAEven ? 0 : (D2 ? cy : cz));
+        const double *p = part + ((int64_t)q * P.nsum + from) * chunks;
 #pragma unroll 8
         for (int c = 0; c < chunks; ++c) s += p[c];
     }
@@ -175,7 +203,7 @@ __global__ void __launch_bounds__(128) k_unit_means(const double *__restrict__ p
     // lane a writes value a (FP64 divisions are slow: one per lane)
     const double v = (i == 0 ? t[0] : (i == 1 ? t[1] : (i == 2 ? t[2] : t[3]))) / (double)M;
     if (i == 0) out[u] = rho0 + v;
-    else if (i < 4) out[units + 3 * u + i - 1] = v;
+    else if (i < 4) out[P.n + 3 * u + i - 1] = v;
 }
 
 }  // namespace profile
@@ -188,26 +216,26 @@ inline int profile_chunks(int64_t M, int units, int nq)
     return (int)(want < most ? want : (most < 1 ? 1 : most));
 }
 
-// The means of every unit of a box (d2: D2Q9): part is scratch of nq units
-// chunks doubles, out receives 4 units doubles.  Units of fewer than 2048
-// elements are summed by one warp each.
+// The means of the units of one pass over a box (d2: D2Q9): part is scratch of nq
+// nsum chunks doubles, out receives 4 n doubles.  Units of fewer than 2048 elements
+// are summed by one warp each.
 template <class S>
-cudaError_t launch_profile(const S *buf, int64_t plane, int layout, int64_t M, int units, bool d2, double rho0,
-                           double *part, double *out, cudaStream_t st)
+cudaError_t launch_profile(const S *buf, int64_t plane, int layout, int64_t M, int units, const profile::Pass &P, bool d2,
+                           double rho0, double *part, double *out, cudaStream_t st)
 {
     const int nq = d2 ? 9 : Q, chunks = profile_chunks(M, units, nq);
-    const int64_t items = (int64_t)units * nq * chunks;
+    const int64_t items = (int64_t)P.nsum * nq * chunks;
     constexpr int T = profile::kThreads;
     if (M < 2048)
-        profile::k_unit_sums<S, 32><<<(unsigned)((items + T / 32 - 1) / (T / 32)), T, 0, st>>>(buf, plane, M, units,
+        profile::k_unit_sums<S, 32><<<(unsigned)((items + T / 32 - 1) / (T / 32)), T, 0, st>>>(buf, plane, M, units, P,
                                                                                                items, chunks, part);
     else
-        profile::k_unit_sums<S, T><<<(unsigned)items, T, 0, st>>>(buf, plane, M, units, items, chunks, part);
+        profile::k_unit_sums<S, T><<<(unsigned)items, T, 0, st>>>(buf, plane, M, units, P, items, chunks, part);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int blocks = (units + 3) / 4;
-    if (d2) profile::k_unit_means<true><<<blocks, 128, 0, st>>>(part, layout, M, units, chunks, rho0, out);
-    else profile::k_unit_means<false><<<blocks, 128, 0, st>>>(part, layout, M, units, chunks, rho0, out);
+    const int blocks = (P.n + 3) / 4;
+    if (d2) profile::k_unit_means<true><<<blocks, 128, 0, st>>>(part, layout, M, P, chunks, rho0, out);
+    else profile::k_unit_means<false><<<blocks, 128, 0, st>>>(part, layout, M, P, chunks, rho0, out);
     return cudaGetLastError();
 }
 

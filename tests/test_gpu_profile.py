@@ -86,3 +86,18 @@ def test_profile_of_more_than_2_to_27_rows():
     want_rho, want_j = reference(n.transpose(2, 0, 1), True)
     # as in the test above
     assert np.abs(rho[rows] - want_rho).max() <= 2e-14 and np.abs(j[:, rows] - want_j).max() <= 2e-14
+
+
+@pytest.mark.parametrize("units", [65536, 65537, 131072 + 5])
+@pytest.mark.parametrize("pattern,steps", [("ab", 2), ("aa", 2), ("aa", 3)])
+@pytest.mark.parametrize("two", [False, True])
+def test_profile_of_several_passes(two, pattern, steps, units):
+    """Boxes of more units than one pass takes: the ends of the passes and of the box."""
+    cfg = flb.config(3, units if two else 1, 1 if two else units, kT=1e-3, gamma_shear=0.3, seed=2, pattern=pattern,
+                     lattice="d2q9" if two else "d3q19")
+    with flb.flb_create_ex(cfg) as ctx:
+        ctx.flb_step(steps)
+        rho, j = ctx.flb_z_profile()
+        want_rho, want_j = reference(ctx.flb_get_populations(), two)
+    # as in the first test
+    assert np.abs(rho - want_rho).max() <= 2e-14 and np.abs(j - want_j).max() <= 2e-14

@@ -71,3 +71,28 @@ def test_row_exchange_slots_lie_in_the_arrays_and_pair_up(tmp_path, xch):
             }}
     if (bad) printf("%d\\n", bad);
     return bad != 0;""", "kernels.cuh")
+
+
+@pytest.mark.parametrize("units", [1, 2, 3, 65535, 65536, 65537, 65538, 131073, 2 ** 29 + 1, 2 ** 31 - 1])
+def test_passes_of_the_plane_averages_cover_every_unit(tmp_path, units):
+    """Each unit is a mean of one pass; slot i's sum that goes into unit u is that of unit u - c_i (periodic)."""
+    run_host(tmp_path, f"""
+    const long long units = {units};
+    long long done = 0;
+    for (long long u0 = 0, k = 0; u0 < units; ++k) {{
+        const profile::Pass p = profile::pass_from((int)u0, (int)units);
+        if (p.n < 1 || p.nsum > profile::kPassUnits + 2) return 1;
+        const bool look = k < 3 || u0 + 3ll * profile::kPassUnits > units;      // the first and last passes, whole
+        for (int m = 0; m < p.n; m += look ? 1 : 32767)
+            for (int shift = -1; shift <= 1; ++shift) {{
+                const int s = profile::sum_of_mean(p, m, shift);
+                const long long want = (u0 + m - shift + units) % units;
+                if (s < 0 || s >= p.nsum || profile::unit_of_sum(p, s, (int)units) != want) {{
+                    printf("unit %lld shift %d: sum %d\\n", u0 + m, shift, s);
+                    return 1;
+                }}
+            }}
+        done += p.n;
+        u0 += p.n;
+    }}
+    return done != units;""", "profile.cuh")
