@@ -318,8 +318,9 @@ int flb_save(flb_ctx *ctx, const char *path);
 int flb_load(flb_ctx *ctx, const char *path);
 
 /* Launch configuration in use, and a measured choice: flb_autotune times every
- * candidate (sites per thread x block shape) for `trials` steps each on the
- * context's own state (which it restores afterwards) and keeps the fastest. */
+ * candidate (sites per thread x block shape; the shape in use and the automatic
+ * ones among them) for `trials` steps each on the context's own state (which it
+ * restores afterwards) and keeps the fastest. */
 int flb_get_launch(const flb_ctx *ctx, int *sites_per_thread, int *block_x, int *block_y);
 /* Sets the launch shape (for instance one that flb_autotune chose earlier for
  * the same boxes); FLB_EINVAL if it does not fit the boxes (sites per thread

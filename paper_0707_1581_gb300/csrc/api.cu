@@ -19,6 +19,7 @@
 #include "d2q9.cuh"
 #include "diag_kernels.cuh"
 #include "kernels.cuh"
+#include "launch_shape.h"
 #include "profile.cuh"
 
 using namespace flb;
@@ -723,130 +724,20 @@ cudaError_t stats_box(flb_ctx *c, Box &b, int layout)
     }
 }
 
-// Largest usable sites-per-thread <= V: the vector path needs nx % V == 0 in
-// every box, at most 16-byte accesses (FP64: V <= 2) and whole warps (its
-// neighbour exchange is a full-warp shuffle), i.e. bx * by % 32 == 0.
-int usable_V(const flb_ctx *c, int V, int bx, int by)
+LaunchBoxes launch_boxes(const flb_ctx *c)
 {
-    if ((bx * by) % 32 != 0) return 1;
-    if (c->store == FLB_STORE_F64 && V > 2) V = 2;
-    for (;;) {
-        bool ok = true;
-        for (const Box &b : c->boxes) ok = ok && (b.cfg.nx % V == 0);
-        if (ok || V == 1) return V;
-        V /= 2;
+    LaunchBoxes B{c->store, is_d2(c), {}, 0};
+    for (const Box &b : c->boxes) {
+        B.nx.push_back(b.cfg.nx);
+        B.sites += b.N;
     }
-}
-
-// Which exchange the single-box kernel uses for a launch shape (measured, see
-// Exchange in kernels.cuh): rows that tile the warps; as many whole rows as the
-// block's threads hold -- FP32 always, the formats bound by instructions (16-bit,
-// FP64) where hardly a lane idles --; blocks that lie in one row where they cover
-// it with few idle lanes; else threads over the whole box.
-void set_exchange(const flb_ctx *c, Launch &L)
-{
-    L.warprow = L.edgerow = false;
-    L.rows = 0;
-    if (c->boxes.size() != 1 || L.V < 2 || is_d2(c)) return;
-    const int V = (c->store == FLB_STORE_F64 && L.V == 4) ? 2 : L.V;
-    const int nx = c->boxes[0].cfg.nx, T = L.bx * L.by;
-    const int g = nx / V;
-    if (L.bx == g && 32 % g == 0 && T % 32 == 0) {
-        L.warprow = true;
-        return;
-    }
-    if (T >= g) {
-        const int rows = std::min(T / g, kXchRows);
-        const double busy = (double)rows * g / ((rows * g + 31) / 32 * 32);
-        if (c->store == FLB_STORE_F32 || busy >= (V == 4 ? 1.0 : 0.95)) {
-            L.rows = rows;
-            return;
-        }
-    }
-    L.edgerow = L.by == 1 && g >= 0.95 * ((g + T - 1) / T * T);
-}
-
-// The block of whole rows of g threads (g <= 256) that keeps most threads busy:
-// the share of its threads that own sites, times the warps an SM holds of it (at
-// 128 registers a thread, 512 threads) over 16.  96 wide (g = 24): 96 threads,
-// 35.0 GLUPS (FP32, AB) against 29.8 with 128 threads of 32 per row.
-int row_block(int g)
-{
-    int best = (g + 31) / 32 * 32;
-    double top = 0.0;
-    for (int rows = 1; rows <= kXchRows && rows * g <= 256; ++rows) {
-        const int T = (rows * g + 31) / 32 * 32;
-        const double busy = (double)rows * g / T * (512 / T * T / 512.0);
-        if (busy > top + 1e-9) {
-            top = busy;
-            best = T;
-        }
-    }
-    return best;
+    return B;
 }
 
 void default_launch(flb_ctx *c)
 {
-    int maxnx = 1;
-    for (const Box &b : c->boxes) maxnx = std::max(maxnx, b.cfg.nx);
     const flb_config &f = c->boxes[0].cfg;
-    Launch L;
-    if (is_d2(c)) {
-        // warps along x, 256 threads; 4 sites per thread (2 for FP64) when nx allows
-        int bx = 32;
-        while (bx < maxnx && bx < 128) bx *= 2;
-        L.bx = f.block_x ? f.block_x : bx;
-        L.by = f.block_y ? f.block_y : std::max(1, 256 / L.bx);
-        const int want = f.sites_per_thread ? f.sites_per_thread : (c->store == FLB_STORE_F64 ? 2 : 4);
-        L.V = usable_V(c, want, L.bx, L.by);
-        if (L.V == 2 && c->store != FLB_STORE_F64) L.V = 1;   // the D2Q9 vector kernel has V = 4 (FP64: 2)
-        c->L = L;
-        return;
-    }
-    int want = f.sites_per_thread ? f.sites_per_thread : (c->store == FLB_STORE_F64 ? 2 : 4);
-    if (!f.sites_per_thread) {
-        // small boxes: fewer sites per thread until there are threads enough to
-        // fill the GPU (~100k: 152 SMs x ~650), measured best for 32^3 and 64^3
-        int64_t total = 0;
-        for (const Box &b : c->boxes) total += b.N;
-        while (want > 1 && total / want < 100000) want /= 2;
-    }
-    if (c->store == FLB_STORE_F64) want = std::min(want, 2);
-    const int sites = (maxnx + want - 1) / want;
-    int bx = 32, by = 0;
-    while (bx < sites && bx < 128) bx *= 2;
-    if (c->boxes.size() == 1) {
-        const Box &b = c->boxes[0];
-        int V = want;
-        while (maxnx % V != 0) V /= 2;
-        const int g = maxnx / V;
-        if (V > 1 && g <= 32 && 32 % g == 0) {
-            bx = g;          // several rows per warp
-        } else if (!f.block_x && !f.block_y) {
-            by = 1;
-            if (V > 1) {
-                Launch r;
-                r.V = V;
-                r.by = 1;
-                r.bx = g <= 256 ? row_block(g) : 128;
-                set_exchange(c, r);
-                // blocks of one row each, of 64 to 160 threads
-                for (int nb = (g + 159) / 160; !r.rows && (nb == (g + 159) / 160 || !r.edgerow) && (g + nb - 1) / nb >= 64; ++nb) {
-                    r.bx = ((g + nb - 1) / nb + 31) / 32 * 32;
-                    set_exchange(c, r);
-                }
-                bx = r.rows || r.edgerow ? r.bx : 128;
-            }
-            // FP64 occupies the SM's FP64 unit 64 cycles per warp instruction: one-warp blocks spread a small
-            // box over the SMs (16^3: 7.8 us per step, 9.1 with 128 threads; 32^3: 14.0, 16.1)
-            else bx = c->store == FLB_STORE_F64 && b.N < 100000 ? 32 : 128;
-        }
-    }
-    L.bx = f.block_x ? f.block_x : bx;
-    L.by = f.block_y ? f.block_y : (by ? by : std::max(1, 128 / L.bx));
-    L.V = usable_V(c, want, L.bx, L.by);
-    set_exchange(c, L);
-    c->L = L;
+    c->L = automatic_launch(launch_boxes(c), f.sites_per_thread, f.block_x, f.block_y);
 }
 
 void free_box(flb_ctx *c, Box &b)
@@ -1749,8 +1640,6 @@ int tune_shapes(flb_ctx *c, int trials, float *best_out)
     if (!c) return FLB_EINVAL;
     if (trials < 1) trials = 1;
     const int nb = (int)c->boxes.size();
-    int maxnx = 1;
-    for (const Box &b : c->boxes) maxnx = std::max(maxnx, b.cfg.nx);
     // back up every box's current state (device to device) and the step counter
     std::vector<void *> backup(nb, nullptr);
     for (int i = 0; i < nb; ++i) {
@@ -1773,37 +1662,26 @@ int tune_shapes(flb_ctx *c, int trials, float *best_out)
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    const int Vs[3] = {1, 2, 4};
-    const int shapes[9][2] = {{32, 4}, {64, 2}, {64, 4}, {128, 1}, {128, 2}, {256, 1}, {16, 8}, {16, 16}, {32, 8}};
-    int rc = FLB_OK;
-    for (int vi = 0; vi < 3 && rc == FLB_OK; ++vi) {
-        for (int si = 0; si < 9 && rc == FLB_OK; ++si) {
-            Launch L;
-            L.V = Vs[vi];
-            L.bx = shapes[si][0];
-            L.by = shapes[si][1];
-            if (usable_V(c, L.V, L.bx, L.by) != L.V) continue;
-            // the D2Q9 vector kernel has one width per format
-            if (is_d2(c) && L.V != 1 && L.V != (c->store == FLB_STORE_F64 ? 2 : 4)) continue;
-            set_exchange(c, L);
-            if (L.bx * L.V > 2 * std::max(32, maxnx)) continue;   // mostly idle threads
-            c->L = L;
-            if ((rc = refresh_batch_tables(c)) != FLB_OK) break;
-            rc = flb_step(c, 2);   // warm-up
-            if (rc != FLB_OK) break;
-            cudaEventRecord(e0, c->stream);
-            rc = flb_step(c, 2 * trials);
-            cudaEventRecord(e1, c->stream);
-            if (cudaEventSynchronize(e1) != cudaSuccess) {
-                rc = cuda_fail(c, cudaGetLastError(), "autotune");
-                break;
-            }
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best_ms) {
-                best_ms = ms;
-                best = L;
-            }
+    int rc = flb_step(c, 2 * trials);   // the clocks are up before the first candidate, the shape in use
+    for (const Launch &L : launch_candidates(launch_boxes(c), keep)) {
+        if (rc != FLB_OK) break;
+        c->L = L;
+        if ((rc = refresh_batch_tables(c)) != FLB_OK) break;
+        rc = flb_step(c, 2);   // warm-up
+        if (rc != FLB_OK) break;
+        cudaEventRecord(e0, c->stream);
+        rc = flb_step(c, 2 * trials);
+        cudaEventRecord(e1, c->stream);
+        if (cudaEventSynchronize(e1) != cudaSuccess) {
+            rc = cuda_fail(c, cudaGetLastError(), "autotune");
+            break;
+        }
+        if (rc != FLB_OK) break;
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (ms < best_ms) {
+            best_ms = ms;
+            best = L;
         }
     }
     cudaEventDestroy(e0);
@@ -1905,14 +1783,15 @@ int flb_set_launch(flb_ctx *c, int V, int bx, int by)
     if (!c) return FLB_EINVAL;
     if ((V != 1 && V != 2 && V != 4) || bx < 1 || by < 1 || bx * by > 256)
         return fail(c, FLB_EINVAL, "sites per thread must be 1, 2 or 4 and block_x * block_y at most 256");
-    if (usable_V(c, V, bx, by) != V) return fail(c, FLB_EINVAL, "this launch shape does not fit the boxes");
+    const LaunchBoxes B = launch_boxes(c);
+    if (usable_V(B, V, bx, by) != V) return fail(c, FLB_EINVAL, "this launch shape does not fit the boxes");
     if (is_d2(c) && V != 1 && V != (c->store == FLB_STORE_F64 ? 2 : 4))
         return fail(c, FLB_EINVAL, "the D2Q9 vector kernel takes 4 sites per thread (2 for FP64)");
     Launch L;
     L.V = V;
     L.bx = bx;
     L.by = by;
-    set_exchange(c, L);
+    set_exchange(B, L);
     c->L = L;
     drop_graphs(c);
     return refresh_batch_tables(c);

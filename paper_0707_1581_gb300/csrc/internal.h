@@ -24,6 +24,8 @@ constexpr int kAccFirst = 28;       // mass, jx, jy, jz at the first sample
 constexpr int kAccLast = 32;        // mass, jx, jy, jz at the last sample
 constexpr int kAccWidth = 36;
 
+constexpr int kXchRows = 32;        // whole rows per block, at most (the exchange memory in kernels.cuh)
+
 // Launch shape of the stream-collide kernels.
 struct Launch {
     int V = 1;        // x-consecutive sites per thread

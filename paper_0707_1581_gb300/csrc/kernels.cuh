@@ -294,14 +294,13 @@ __device__ __forceinline__ R shfl_down1(R v)
 // instructions, only where no lane idles: 300 x 200 x 60 AB 61.7 / 66.3, 400 x
 // 100 x 100 64.5 / 76.1 (kRagRow, 100 of 128 lanes), 640 wide 132 / 129; two sites
 // per thread 87 / 77 (250 wide AA).  FP64 likewise: 90 x 100 x 110 368 / 397 (90 of
-// 96 lanes), 72^3 154 / 145.  (set_exchange in api.cu decides.)
+// 96 lanes), 72^3 154 / 145.  (set_exchange in launch_shape.h decides.)
 enum Exchange : int { kEdges = 0, kOneRow = 1, kRows = 2, kWarpRow = 3, kRagRow = 4, kEdgeRow = 5 };
 
 // The block's exchange memory: what a warp (kOneRow) or a warp or row (kRows)
 // hands over its ends, in the load phase (l*, as stored) and in the store phase
 // (s*).
-constexpr int kXchWarps = 8;       // warps per block, at most
-constexpr int kXchRows = 32;       // rows per block, at most
+constexpr int kXchWarps = 8;       // warps per block, at most (rows: kXchRows)
 template <class S, int XCH>
 struct RowExchange {
     using R = typename Storage<S>::R;
