@@ -417,8 +417,9 @@ int upload_batch_tables(flb_ctx *c)
             BoxStep<S> s = make_step<S>(c, b, o);
             const int T = c->L.bx * c->L.by, g = s.groups;
             s.warprow = c->L.V > 1 && g <= 32 && 32 % g == 0;
-            // FP32: whole rows per block; else threads packed densely over the box
-            if (c->L.V > 1 && sizeof(S) == 4 && !s.warprow && g <= T) s.rows = std::min(T / g, kXchRows);
+            // FP32: whole rows per block where they fill it; else threads packed densely over the box
+            if (c->L.V > 1 && sizeof(S) == 4 && !s.warprow)
+                s.rows = batch_rows(g, T, c->L.V, c->pattern == FLB_PATTERN_AA);
             const int64_t rows = (int64_t)b.cfg.ny * b.cfg.nz;
             s.block0 = blocks;
             blocks += (int)(s.rows ? (rows + s.rows - 1) / s.rows : (rows * g + T - 1) / T);

@@ -684,9 +684,9 @@ __global__ void __launch_bounds__(256, kMinBlocks<S, V, XCH>) k_stream_collide(c
 }
 
 // Many boxes in one 1-D grid: box b owns the blocks from block0 on.  FP32 boxes
-// whose rows do not tile the warps take whole rows per block (kRows: 12 boxes of
-// 96^3, AB, 45.5 GLUPS against 39.9 with the scalar accesses of kEdges); in the
-// other boxes the threads are packed densely: thread item k = (block - block0) T
+// whose rows do not tile the warps but nearly fill the blocks (batch_rows) take whole
+// rows per block (kRows: 12 boxes of 96^3, AB, 45.3 GLUPS against 41.0 with the scalar
+// accesses of kEdges); in the other boxes the threads are packed densely: thread item k = (block - block0) T
 // + tid owns the V sites of x-group k mod groups (nx / V groups per row) of row k
 // / groups, so a warp may span several short rows and no lane idles at a row
 // end.  The box table is a kernel parameter (constant bank, at most ~31 KB);

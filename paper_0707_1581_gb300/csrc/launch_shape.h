@@ -82,6 +82,29 @@ inline int row_block(int g)
     return best;
 }
 
+// Whole rows per block of an FP32 box of a batch, whose blocks of T threads serve
+// boxes of every width: T / g rows of g threads where the threads that are left
+// over cost less than the whole-row exchange gains over threads packed densely
+// over the box (0: packed).  They cost their share of the SM's threads, more so in
+// large blocks, of which the SM holds few; the exchange gains most for AA steps
+// with four sites per thread, which have the most scalar accesses without it.  The
+// line is where both ran equal, 8 boxes of 0.75 M sites, 10 to 34 widths for each T
+// (whole rows / packed at a busy share of 0.66, 0.75, 0.84, 0.94):
+//   AB V = 4, T 128  0.91 0.98 1.06 1.11   T 256  0.82 0.89 0.94 1.00
+//   AB V = 2, T 128  0.93 1.02 1.12 1.20   T 256  0.91 1.00 1.06 1.14
+//   AA V = 4, T 128  0.99 1.08 1.15 1.22   T 256  0.92 1.00 1.06 1.14
+//   AA V = 2, T 128  0.85 0.93 1.00 1.06   T 256  0.83 0.91 0.96 1.04
+// Blocks of one warp gain nothing.  A batch of 264-wide boxes (66 of 128 threads
+// busy with whole rows), AB: 29.5 GLUPS with whole rows, 40.8 packed.
+inline int batch_rows(int g, int T, int V, bool aa)
+{
+    if (g > T || T < 64) return 0;
+    const int rows = std::min(T / g, kXchRows);
+    double least = aa ? (V == 4 ? 0.70 : 0.86) : (V == 4 ? 0.78 : 0.76);
+    if (T > 128) least += (T - 128) / 128.0 * (aa ? (V == 4 ? 0.09 : 0.05) : (V == 4 ? 0.17 : 0.05));
+    return (double)rows * g / T >= least ? rows : 0;
+}
+
 // The shape for what a caller leaves open (sites_per_thread, block_x, block_y; 0 = open).
 inline Launch automatic_launch(const LaunchBoxes &B, int sites_per_thread, int block_x, int block_y)
 {

@@ -63,3 +63,23 @@ def test_automatic_shapes_outside_the_fixed_blocks_are_candidates(tmp_path):
         for (const Launch &L : launch_candidates(B, now)) n += L.V == a.V && L.bx == a.bx && L.by == a.by;
         printf("%d %d %d %d\\n", a.V, a.bx, a.by, n);
     }""", "launch_shape.h").split() == "1 32 1 1 4 96 1 1 4 160 1 1".split()
+
+
+def test_whole_rows_of_a_batch_leave_few_threads_idle(tmp_path):
+    """Boxes of a batch take whole rows only where they fill the blocks: rows of 66, 80 and 96 threads in blocks of
+    128, or of 3 in blocks of 256 (at most 32 rows), are packed densely; 24, 32 - 1 and 127 keep whole rows."""
+    run_host(tmp_path, """
+    for (int aa = 0; aa < 2; ++aa)
+        for (int V : {2, 4})
+            for (int T = 32; T <= 256; T += 32)
+                for (int g = 1; g <= 1024; ++g) {
+                    const int r = batch_rows(g, T, V, aa != 0);
+                    if (r < 0 || r > kXchRows || r * g > T) return 1;
+                    if (r && r * g < 0.7 * T) return 2;              // idle threads
+                    if (T >= 64 && g <= T && r == 0 && std::min(T / g, kXchRows) * g >= 0.96 * T) return 3;
+                }
+    for (int g : {66, 80}) if (batch_rows(g, 128, 4, false) || batch_rows(g, 128, 4, true)) return 4;
+    if (batch_rows(96, 128, 4, false) || batch_rows(3, 256, 4, false) || batch_rows(3, 256, 4, true)) return 5;
+    if (batch_rows(24, 128, 4, false) != 5 || batch_rows(31, 128, 4, false) != 4 || batch_rows(127, 128, 4, true) != 1)
+        return 6;
+    return 0;""", "launch_shape.h")
