@@ -15,14 +15,52 @@ int grid_for(int64_t n, int threads)
     return g < 1 ? 1 : (int)g;
 }
 
+// When a step of the one-site kernel lets the next one start, as start_point below:
+// at the start in boxes of up to half a block per SM and of many waves, whose blocks
+// do not crowd onto few SMs; in between after the loads, or before the stores where
+// the in-place steps and the stochastic format, with more to do between the two, would
+// still crowd; FP64, whose unit is the bound, before the stores.  us per step, unchained
+// / at the start / after the loads / before the stores, plain launches (graphs):
+//   FP64 AB   51 x 301 (76 blocks)   10.27 / 17.78 /  8.31 /  8.61   (9.04 / 8.65 / 8.43 / 8.63)
+//             117 x 300 (150)        10.56 / 26.37 /  8.41 /  8.66   (9.24 / 13.2 / 8.62 / 8.65)
+//             301 x 301 (453)        24.62 / 29.42 / 29.37 / 22.64   (23.2 / 28.9 / 28.9 / 22.8)
+//   FP16 AB   301 x 301               5.07 /  4.46 /  2.39 /  2.73   (3.30 / 3.45 / 2.70 / 2.70)
+//             401 x 301 (604)         6.18 /  4.01 /  2.85 /  3.36   (3.94 / 3.90 / 3.12 / 3.52)
+//             1001 x 601 (2408)      11.91 /  8.80 /  8.76 /  9.23   (9.89 / 8.99 / 8.87 / 9.28)
+//   FP16 AA   301 x 301               4.64 /  3.03 /  2.63 /  2.62   (3.10 / 3.11 / 3.03 / 2.67)
+//   stochastic AB  301 x 301          6.17 /  5.53 /  3.37 /  3.17   (3.72 / 4.26 / 3.52 / 3.31)
+//             117 x 300               4.12 /  2.63 /  2.12 /  2.31   (2.69 / 2.25 / 2.49 / 2.28)
+template <class S, int LAYOUT>
+StartPoint start_point_one(int64_t blocks, bool in_graph)   // of 256 threads
+{
+    constexpr int64_t kSMs = 152;
+    if (sizeof(S) == 8) return blocks <= kSMs / 2 ? kAfterLoads : kBeforeStores;
+    if (blocks <= kSMs) return in_graph || blocks <= kSMs / 2 ? kAtStart : kAfterLoads;
+    if (blocks > 6 * kSMs) return kAtStart;
+    return LAYOUT == kAB && !Storage<S>::stochastic ? kAfterLoads : kBeforeStores;
+}
+
+template <class S, int LAYOUT, bool NOISE, bool FORCE>
+cudaError_t step_one(const BoxStep<S> &b, dim3 grid, dim3 block, const uint32_t *p, uint32_t t, cudaStream_t st)
+{
+    const StartPoint at = start_point_one<S, LAYOUT>((int64_t)grid.x * block.x * block.y / 256, p != nullptr);
+    if constexpr (sizeof(S) < 8) {
+        if (at == kAtStart)
+            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, kAtStart>, grid, block, st, b, p, t);
+    }
+    if (at == kBeforeStores)
+        return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, kBeforeStores>, grid, block, st, b, p, t);
+    return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, kAfterLoads>, grid, block, st, b, p, t);
+}
+
 template <class S, int LAYOUT>
 cudaError_t step_layout(const BoxStep<S> &b, bool noise, bool force, dim3 grid, dim3 block, const uint32_t *p,
                         uint32_t t, cudaStream_t st)
 {
-    if (noise && force) return launch_chained(k_stream_collide<S, LAYOUT, true, true>, grid, block, st, b, p, t);
-    if (noise) return launch_chained(k_stream_collide<S, LAYOUT, true, false>, grid, block, st, b, p, t);
-    if (force) return launch_chained(k_stream_collide<S, LAYOUT, false, true>, grid, block, st, b, p, t);
-    return launch_chained(k_stream_collide<S, LAYOUT, false, false>, grid, block, st, b, p, t);
+    if (noise && force) return step_one<S, LAYOUT, true, true>(b, grid, block, p, t, st);
+    if (noise) return step_one<S, LAYOUT, true, false>(b, grid, block, p, t, st);
+    if (force) return step_one<S, LAYOUT, false, true>(b, grid, block, p, t, st);
+    return step_one<S, LAYOUT, false, false>(b, grid, block, p, t, st);
 }
 
 // V sites per thread: 16-byte accesses for 4-byte formats, 8-byte for 16-bit, V = 2 for FP64.

@@ -203,11 +203,12 @@ struct BoxStep {
 //   AB      pull n_i(r) from slot i at r - c_i of src, store n*_i(r) in slot i at r of dst.
 //   AA even read slot i at r, store n*_i(r) in slot opposite(i) at r.
 //   AA odd  read slot opposite(i) at r - c_i, store n*_i(r) in slot i at r + c_i.
-template <class S, int LAYOUT, bool NOISE, bool FORCE>
+// START: when a step's blocks let the next step's start (start_point_one in d2q9.cu has the rule)
+template <class S, int LAYOUT, bool NOISE, bool FORCE, int START>
 __global__ void __launch_bounds__(256) k_stream_collide(const BoxStep<S> B, const uint32_t *step_ptr, uint32_t step)
 {
     using R = typename Storage<S>::R;
-    let_next_step_start();
+    if constexpr (START == kAtStart) let_next_step_start();
     const int bxi = blockIdx.x % B.gx, byi = blockIdx.x / B.gx;
     const int x = bxi * blockDim.x + threadIdx.x;
     const int y = byi * blockDim.y + threadIdx.y;
@@ -233,10 +234,12 @@ __global__ void __launch_bounds__(256) k_stream_collide(const BoxStep<S> B, cons
         const S *p = B.src + (int64_t)slot * B.plane + idx;
         f[i] = Storage<S>::load(load_ro(FLB_GUARD_LD(B, p, 1)));
     }
+    if constexpr (START == kAfterLoads) let_next_step_start();
     R Fx = R(0);
     if (FORCE) Fx = B.K.force_amp * sin_pi(B.K.force_phase * R(y));
     collide<R, NOISE, FORCE>(f, B.K, (uint32_t)site, step, B.replica, Fx);
     stochastic_round<S>(f, (uint32_t)site, step, B.replica, B.K.rk0, B.K.rk1);
+    if constexpr (START == kBeforeStores) let_next_step_start();
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         int idx = site, slot = i;

@@ -182,3 +182,19 @@ def test_chained_d2q9_steps_equal_steps_one_at_a_time(pattern, graph_steps, stor
     with flb.flb_create_ex(box(nx, ny, 1, store, pattern, graph_steps=graph_steps, **cfg)) as ctx:
         ctx.flb_step(21)
         assert np.array_equal(raw(ctx), want)
+
+
+@pytest.mark.parametrize("nx,ny", [(7, 9), (51, 301), (117, 300), (301, 301), (501, 601), (1001, 601)])
+@pytest.mark.parametrize("store", ["f64", "f32", "bf16dev", "bf16sr"])
+@pytest.mark.parametrize("pattern,graph_steps", [("ab", 0), ("aa", 0), ("ab", 10), ("aa", 10)])
+def test_chained_one_site_d2q9_steps_equal_steps_one_at_a_time(pattern, graph_steps, store, nx, ny):
+    """Odd rows: every start point of the one-site kernel (half a block per SM, one, several, many)."""
+    cfg = dict(lattice="d2q9", kT=1e-4, force_amp=1e-5)
+    with flb.flb_create_ex(box(nx, ny, 1, store, pattern, **cfg)) as ctx:
+        for _ in range(21):
+            ctx.flb_step(1)
+            ctx.flb_sync()
+        want = raw(ctx)
+    with flb.flb_create_ex(box(nx, ny, 1, store, pattern, graph_steps=graph_steps, **cfg)) as ctx:
+        ctx.flb_step(21)
+        assert np.array_equal(raw(ctx), want)
