@@ -84,12 +84,19 @@ constexpr int vec_width()
 //   FP32  236 x 551               6.19 / 6.27 / 3.45 / 3.53
 //         752 x 437 (321)         8.24 / 7.37 / 6.39 / 5.47
 //         1744 x 864 (1472)       18.49 / 16.08 / 17.10 / 16.24;  3000 x 2400  86.9 / 86.2 / 78.1 / 84.9
-template <class S, int LAYOUT>
+// FP64 waits for its loads, but for AB steps without a force of 1.5 to 2 blocks per SM:
+// those kernels leave room for three blocks on an SM, so some SMs get three while others
+// hold one; the other FP64 kernels leave room for two.
+//   FP64 AB  256 x 456 (228 blocks)  32.80 / - / 30.23 / 30.16; in graphs 30.75 / - / 30.40 / 31.09
+//            256 x 480 (240)         32.80 / - / 44.08 / 30.69; in graphs 30.78 / - / 43.07 / 32.28
+//            256 x 600 (300)         32.82 / - / 44.23 / 35.79;  256 x 612 (306)  47.13 / - / 44.26 / 44.00
+template <class S, int LAYOUT, bool FORCE>
 StartPoint start_point(const BoxStep<S> &b, int64_t blocks, bool in_graph)   // of 256 threads
 {
     constexpr int64_t kSMs = 152;
     constexpr int64_t kL2 = 128000000;
-    if (sizeof(S) == 8) return kAfterLoads;
+    if (sizeof(S) == 8)
+        return LAYOUT == kAB && !FORCE && 2 * blocks > 3 * kSMs && blocks <= 2 * kSMs ? kUnchained : kAfterLoads;
     if (sizeof(S) == 2) return blocks <= kSMs ? kAfterLoads : blocks <= 2 * kSMs ? kBeforeStores : kAtStart;
     const bool in_l2 = (LAYOUT == kAB ? 2 : 1) * Q * b.plane * (int64_t)sizeof(S) <= kL2;
     // a graph's launches are close enough for a state in L2: 632 x 640 FP32 takes 5.82 us
@@ -102,7 +109,7 @@ template <class S, int LAYOUT, bool NOISE, bool FORCE>
 cudaError_t step_vec(const BoxStep<S> &b, dim3 grid, dim3 block, const uint32_t *p, uint32_t t, cudaStream_t st)
 {
     constexpr int V = vec_width<S>();
-    const StartPoint at = start_point<S, LAYOUT>(b, (int64_t)grid.x * block.x * block.y / 256, p != nullptr);
+    const StartPoint at = start_point<S, LAYOUT, FORCE>(b, (int64_t)grid.x * block.x * block.y / 256, p != nullptr);
     if constexpr (sizeof(S) == 2) {
         if (at == kAtStart)
             return launch_chained(k_stream_collide_vec<S, LAYOUT, NOISE, FORCE, V, kAtStart>, grid, block, st, b, p, t);
@@ -111,9 +118,10 @@ cudaError_t step_vec(const BoxStep<S> &b, dim3 grid, dim3 block, const uint32_t 
         if (at == kBeforeStores)
             return launch_chained(k_stream_collide_vec<S, LAYOUT, NOISE, FORCE, V, kBeforeStores>, grid, block, st, b, p, t);
     }
-    if constexpr (sizeof(S) == 4) {
+    if constexpr (sizeof(S) >= 4) {
         if (at == kUnchained) {
-            k_stream_collide_vec<S, LAYOUT, NOISE, FORCE, V, kBeforeStores><<<grid, block, 0, st>>>(b, p, t);
+            constexpr int kAny = sizeof(S) == 8 ? kAfterLoads : kBeforeStores;
+            k_stream_collide_vec<S, LAYOUT, NOISE, FORCE, V, kAny><<<grid, block, 0, st>>>(b, p, t);
             return cudaGetLastError();
         }
     }

@@ -198,3 +198,22 @@ def test_chained_one_site_d2q9_steps_equal_steps_one_at_a_time(pattern, graph_st
     with flb.flb_create_ex(box(nx, ny, 1, store, pattern, graph_steps=graph_steps, **cfg)) as ctx:
         ctx.flb_step(21)
         assert np.array_equal(raw(ctx), want)
+
+
+@pytest.mark.parametrize("nx,ny,force", [(256, 456, 0.0), (256, 458, 0.0), (256, 608, 0.0), (256, 610, 0.0),
+                                         (256, 480, 1e-5)])
+@pytest.mark.parametrize("pattern,graph_steps", [("ab", 0), ("aa", 0), ("ab", 10)])
+def test_chained_fp64_d2q9_steps_of_two_blocks_per_sm(pattern, graph_steps, nx, ny, force):
+    """On either side of the range of unchained FP64 steps; a statistics sample after them."""
+    cfg = dict(lattice="d2q9", kT=1e-4, force_amp=force)
+    with flb.flb_create_ex(box(nx, ny, 1, "f64", pattern, **cfg)) as ctx:
+        for _ in range(21):
+            ctx.flb_step(1)
+            ctx.flb_sync()
+        ctx.flb_stats_sample()
+        want, stats = raw(ctx), ctx.flb_mode_stats()
+    with flb.flb_create_ex(box(nx, ny, 1, "f64", pattern, graph_steps=graph_steps, **cfg)) as ctx:
+        ctx.flb_step(21)
+        ctx.flb_stats_sample()
+        assert np.array_equal(raw(ctx), want)
+        assert np.array_equal(ctx.flb_mode_stats()["mode_m2"], stats["mode_m2"])
