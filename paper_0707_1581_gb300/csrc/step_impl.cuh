@@ -15,11 +15,15 @@ cudaError_t step_one(const BoxStep<S> &b, const Launch &L, const uint32_t *step_
 {
     const int g = b.nx / V, T = L.bx * L.by;
     if constexpr (V > 1) {
+        // the three-dimensional grids end at 65535 along y and z; longer boxes take the forms with one grid index
+        constexpr int kGridYZ = 65535;
         const bool off32 = (uint64_t)Q * (uint64_t)b.plane < (1ull << 32);
-        if (L.warprow)
-            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, kWarpRow>,
-                                  dim3(1, (b.ny + L.by - 1) / L.by, b.nzl), dim3(L.bx, L.by), st, b, step_ptr, step);
-        if (L.rows == 1 && off32 && b.ny <= 65535) {
+        const bool planes = b.nzl <= kGridYZ, lines = planes && b.ny <= kGridYZ;
+        const int warp_blocks = b.ny / L.by + (b.ny % L.by != 0);
+        if (L.warprow && planes && warp_blocks <= kGridYZ)
+            return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, kWarpRow>, dim3(1, warp_blocks, b.nzl),
+                                  dim3(L.bx, L.by), st, b, step_ptr, step);
+        if (L.rows == 1 && off32 && lines) {
             const dim3 grid(1, b.ny, b.nzl), block((g + 31) / 32 * 32);
             if (g % 32 == 0)
                 return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, kOneRow, true>, grid, block, st, b,
@@ -35,9 +39,7 @@ cudaError_t step_one(const BoxStep<S> &b, const Launch &L, const uint32_t *step_
             return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, kRows>, grid, block, st, r, step_ptr,
                                   step);
         }
-    }
-    if constexpr (V > 1) {
-        if (L.edgerow && b.ny <= 65535)
+        if (L.edgerow && lines)
             return launch_chained(k_stream_collide<S, LAYOUT, NOISE, FORCE, V, kEdgeRow>,
                                   dim3((g + T - 1) / T, b.ny, b.nzl), dim3(T), st, b, step_ptr, step);
     }

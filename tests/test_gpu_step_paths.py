@@ -217,3 +217,24 @@ def test_chained_fp64_d2q9_steps_of_two_blocks_per_sm(pattern, graph_steps, nx, 
         ctx.flb_stats_sample()
         assert np.array_equal(raw(ctx), want)
         assert np.array_equal(ctx.flb_mode_stats()["mode_m2"], stats["mode_m2"])
+
+
+@pytest.mark.parametrize("nx,ny,nz,store", [(16, 1, 70000, "f32"), (16, 2097153, 1, "f32"), (256, 1, 66000, "f32"),
+                                            (250, 1, 66000, "f32"), (250, 66000, 1, "f32"), (1000, 1, 66000, "f16dev"),
+                                            (1000, 66000, 1, "f16dev"), (32, 1, 70000, "f64")])
+def test_boxes_of_more_planes_or_rows_than_a_grid_dimension(nx, ny, nz, store):
+    """Rows that tile the warps, whole rows, blocks inside a row: against the scalar path, at sampled sites."""
+    cfg = box(nx, ny, nz, store, "aa", kT=1e-3, force_amp=1e-3)
+    N = nx * ny * nz
+    sites = np.unique(np.concatenate([[0, N - 1, N - nx, 65535 * nx, min(N - 1, 65536 * nx + nx - 1)],
+                                      np.random.default_rng(1).integers(0, N, 2000)]))
+    got = []
+    for launch in (None, (1, 128, 1)):
+        with flb.flb_create_ex(cfg) as ctx:
+            if launch:
+                ctx.flb_set_launch(*launch)
+            else:
+                assert ctx.flb_get_launch()[0] > 1
+            ctx.flb_step(3)
+            got.append(ctx.flb_get_sites(sites))
+    assert np.abs(got[0] - got[1]).max() <= TOLERANCE[store]
