@@ -5,10 +5,10 @@
 // a population inside its unit do not change the unit's sum, so the sum of the
 // canonical n_i over unit u is the sum of one slot's contiguous unit u - c_i: the
 // first kernel sums every unit of every slot as one stream, the second combines
-// the Q sums of each unit.  Bound by HBM: 512^3 FP32 1.42 ms per call (10.2 GB at
-// 7.2 TB/s), 256^3 bfloat16 0.13 ms; one block per plane with every site's
-// populations added in FP64 took 34.3 and 4.3 ms, 64^3 FP32 160 us (now 28, of
-// which about 20 are the call's launches and wait).
+// the Q sums of each unit.  FP32 is bound by HBM: 512^3 1.40 ms per call (10.2 GB at
+// 7.3 TB/s), 64^3 27 us, of which about 20 are the call's launches and wait; 16-bit
+// formats by the additions (512^3 FP16 1.08 ms, 256^3 bfloat16 0.17).  One block per
+// plane with every site's populations added in FP64 took 34.3 ms, 160 us, 34.2 and 4.3 ms.
 #pragma once
 
 #include "d3q19.cuh"
@@ -17,36 +17,54 @@
 namespace flb {
 namespace profile {
 
-// s + v without a rounding error: the sum and what it lost (Knuth's TwoSum).
+// a + b without a rounding error: the sum and what it lost (Knuth's TwoSum).
 __device__ __forceinline__ float two_sum(float a, float b, float &err)
 {
-    const float s = __fadd_rn(a, b), bb = __fadd_rn(s, -a);
-    err = __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb));
+    const float s = __fadd_rn(a, b), t = __fadd_rn(a, -s);   // -t: what s took of b
+    err = __fadd_rn(__fadd_rn(a, -__fadd_rn(s, t)), __fadd_rn(b, t));
     return s;
 }
 
-// A running sum of 16- or 32-bit values as an unevaluated pair of floats (48
-// bits): an FP64 addition occupies an SM quarter's FP64 unit for 64 cycles per
-// warp, and a conversion to FP64 as long, seven FP32 additions for seven.  A
-// sum that leaves the range of FP32 (or meets an infinity or NaN) shows as a
-// non-finite hi; its values are then summed again in FP64.
-struct PairSum {
-    float hi = 0.f, lo = 0.f;
+// A running sum of 16- or 32-bit values as an unevaluated sum of three floats: an
+// FP64 addition occupies an SM quarter's FP64 unit for 64 cycles per warp, and a
+// conversion to FP64 as long, thirteen FP32 additions for thirteen.  hi takes the
+// values, mid what hi loses, lo what mid loses; settle() passes what has gathered in
+// mid and lo upwards.  With n values between two calls mid is at most n 2^-24 of the
+// largest hi, and an addition to lo rounds by at most 2^-24 n 2^-24 n 2^-24 of it,
+// 2^-61 for n = 40: less than the 2^-53 of an FP64 addition.  A sum that leaves the
+// range of FP32 (or meets an infinity or NaN) shows as non-finite; its values are then
+// summed again in FP64.
+struct TripleSum {
+    float hi = 0.f, mid = 0.f, lo = 0.f;
     __device__ __forceinline__ void add(float v)
     {
-        float e;
+        float e, e2;
         hi = two_sum(hi, v, e);
-        lo += e;
+        mid = two_sum(mid, e, e2);
+        lo += e2;
     }
-    __device__ __forceinline__ void add(PairSum o)
+    __device__ __forceinline__ void add(const TripleSum &o)
     {
+        float e;
         add(o.hi);
-        lo += o.lo;
+        mid = two_sum(mid, o.mid, e);
+        lo += e + o.lo;
     }
+    __device__ __forceinline__ void settle()
+    {
+        float t;
+        hi = two_sum(hi, mid, t);
+        mid = two_sum(t, lo, lo);
+    }
+    __device__ __forceinline__ bool finite() const { return isfinite(hi) && isfinite(mid) && isfinite(lo); }
+    __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
 };
 
-constexpr int kThreads = 256;     // per block
+constexpr int kThreads = 128;     // per block; 16 blocks per SM (32 registers): 512^3 FP32 1.40 ms, 1.75 with what is left
+                                  // free (40); 256 threads take 1.40 ms too, but 64^3 bfloat16 30.6 us against 27.2
 constexpr int kUnroll = 4;        // 16-byte loads in flight per thread
+template <class S>
+constexpr int kSettle = sizeof(S) == 4 ? 8 : 4;   // loads between two calls of settle: 32 values
 
 // The units of one pass: the sums of nsum consecutive units from `first` on (modulo
 // the box's units), then the means of n units, of which the first is the lead-th
@@ -80,7 +98,7 @@ __host__ __device__ inline int sum_of_mean(const Pass &p, int k, int shift)
 // unit_of_sum) of slot q, M elements per unit, into part[(q nsum + u) chunks + c];
 // work item w is (c, q, u) with u fastest.
 template <class S, int T>
-__global__ void __launch_bounds__(kThreads) k_unit_sums(const S *__restrict__ buf, int64_t plane, int64_t M, int units,
+__global__ void __launch_bounds__(kThreads, 16) k_unit_sums(const S *__restrict__ buf, int64_t plane, int64_t M, int units,
                                                         Pass P, int64_t items, int chunks, double *__restrict__ part)
 {
     constexpr int E = 16 / sizeof(S);   // elements per 16-byte load
@@ -98,9 +116,11 @@ __global__ void __launch_bounds__(kThreads) k_unit_sums(const S *__restrict__ bu
     const int64_t head = min(n, (int64_t)((16 - reinterpret_cast<uintptr_t>(p) % 16) % 16 / sizeof(S)));
     const int64_t vecs = (n - head) / E, tail = n - head - vecs * E;
     const uint4 *v = reinterpret_cast<const uint4 *>(p + head);
-    auto each = [&](auto f) {   // f(value, which of two chains)
-        if (tid < head) f(p[tid], 0);
-        if (tid < tail) f(p[head + vecs * E + tid], 1);
+    // f(value), and after(loads) after every kUnroll loads
+    auto each = [&](auto f, auto after) {
+        if (tid < head) f(p[tid]);
+        if (tid < tail) f(p[head + vecs * E + tid]);
+        int loads = 0;
         for (int64_t i0 = tid; i0 < vecs; i0 += kUnroll * T) {
             uint4 x[kUnroll];
 #pragma unroll
@@ -110,38 +130,57 @@ __global__ void __launch_bounds__(kThreads) k_unit_sums(const S *__restrict__ bu
             for (int r = 0; r < kUnroll; ++r) {
                 const S *e = reinterpret_cast<const S *>(&x[r]);
 #pragma unroll
-                for (int k = 0; k < E; ++k) f(e[k], k & 1);
+                for (int k = 0; k < E; ++k) f(e[k]);
             }
+            after(loads += kUnroll);
         }
     };
-    double sum;
-    if constexpr (sizeof(S) == 8) {
-        sum = 0.0;
-        each([&](S x, int) { sum += x; });
+    auto over_lanes = [](double x) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-    } else {
-        PairSum a, b;
-        each([&](S x, int k) {
-            if (k) b.add(Storage<S>::load(x));
-            else a.add(Storage<S>::load(x));
-        });
-        a.add(b);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            PairSum o;
-            o.hi = __shfl_xor_sync(0xffffffffu, a.hi, off);
-            o.lo = __shfl_xor_sync(0xffffffffu, a.lo, off);
-            a.add(o);
+        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+        return x;
+    };
+    double *const to = part + ((int64_t)q * P.nsum + u) * chunks + c;
+    if constexpr (sizeof(S) < 8) {
+        TripleSum s;
+        each([&](S x) { s.add(Storage<S>::load(x)); },
+             [&](int loads) {
+                 if (loads % kSettle<S> == 0) s.settle();
+             });
+        // the first warp adds the block's warps lane by lane, then its lanes
+        __shared__ float all[3][kWarps][32];
+        bool fp64 = !s.finite();
+        if constexpr (kWarps > 1) {
+            all[0][tid / 32][tid % 32] = s.hi;
+            all[1][tid / 32][tid % 32] = s.mid;
+            all[2][tid / 32][tid % 32] = s.lo;
+            fp64 = __syncthreads_or(fp64);
         }
-        sum = (double)a.hi + (double)a.lo;
-        if (__any_sync(0xffffffffu, !isfinite(a.hi) || !isfinite(a.lo))) {
-            sum = 0.0;
-            each([&](S x, int) { sum += Storage<S>::to_double(x); });
+        if (!__any_sync(0xffffffffu, fp64)) {
+            if (tid >= 32) return;
+            auto of = [&](int k) { return TripleSum{all[0][k][tid], all[1][k][tid], all[2][k][tid]}; };
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            for (int k = 1; k < kWarps; ++k) s.add(of(k));
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1)
+                s.add(TripleSum{__shfl_xor_sync(0xffffffffu, s.hi, off), __shfl_xor_sync(0xffffffffu, s.mid, off),
+                                __shfl_xor_sync(0xffffffffu, s.lo, off)});
+            const bool ok = !__any_sync(0xffffffffu, !s.finite());   // else out of range only together
+            if (kWarps > 1 || ok) {
+                double sum = s.value();
+                if (!ok) {
+                    sum = 0.0;
+                    for (int k = 0; k < kWarps; ++k) sum += of(k).value();
+                    sum = over_lanes(sum);
+                }
+                if (tid == 0) *to = sum;
+                return;
+            }
         }
     }
+    double sum = 0.0;
+    each([&](S x) { sum += Storage<S>::to_double(x); }, [](int) {});
+    sum = over_lanes(sum);
     if constexpr (kWarps > 1) {
         __shared__ double wsum[kWarps];
         if ((tid & 31) == 0) wsum[tid >> 5] = sum;
@@ -152,7 +191,7 @@ __global__ void __launch_bounds__(kThreads) k_unit_sums(const S *__restrict__ bu
             for (int k = 0; k < kWarps; ++k) sum += wsum[k];
         }
     }
-    if (tid == 0) part[((int64_t)q * P.nsum + u) * chunks + c] = sum;
+    if (tid == 0) *to = sum;
 }
 
 // The unit of a thread of k_unit_means.  Warps are counted, not threads: 2^27 units have

@@ -1,4 +1,6 @@
 """Plane and row averages (flb_box_z_profile) against sums of the canonical populations."""
+import math
+
 import numpy as np
 import pytest
 
@@ -101,3 +103,39 @@ def test_profile_of_several_passes(two, pattern, steps, units):
         want_rho, want_j = reference(ctx.flb_get_populations(), two)
     # as in the first test
     assert np.abs(rho - want_rho).max() <= 2e-14 and np.abs(j - want_j).max() <= 2e-14
+
+
+@pytest.mark.parametrize("store,w", [("f32", 2.0 ** -26 * (1 + 2.0 ** -22 + 2.0 ** -23)), ("f32", 2.0 ** -27 * 1.7320508),
+                                     ("bf16dev", 2.0 ** -27 * 1.75)])
+def test_profile_keeps_the_bits_of_an_fp64_sum(store, w):
+    """A few ones before many values below their 24 bits: the partial sums have to hold more than 48 bits."""
+    nx = ny = 1024
+    with flb.flb_create_ex(flb.config(nx, ny, 1, store=store, pattern="ab")) as ctx:
+        x = np.full(nx * ny, w, np.float32)
+        if store == "bf16dev":                       # the stored values: bfloat16 bits, of several sizes
+            x[::3] *= 2.0 ** -9
+            x[1::7] *= 2.0 ** -17
+        x[np.arange(nx * ny) % 16384 < 1024] = 1.0
+        raw = np.zeros(ctx.flb_state_bytes(), np.uint8)
+        planes = raw.view(np.float32 if store == "f32" else np.uint16).reshape(19, -1)
+        planes[5, :nx * ny] = x if store == "f32" else x.view(np.uint32) >> 16
+        ctx.flb_state_upload(raw)
+        j = ctx.flb_z_profile()[1]
+    stored = x if store == "f32" else ((x.view(np.uint32) >> 16) << 16).view(np.float32)
+    want = math.fsum(stored.astype(np.float64)) / (nx * ny)
+    # slot 5 moves along z.  At most two roundings per thread, 8 warps, 64 pieces of the plane and the division, each
+    # of 2^-53 of a sum no larger than the total
+    assert abs(j[2, 0] - want) <= 75 * 2.0 ** -53 * want
+
+
+@pytest.mark.parametrize("nx,ny", [(64, 40), (16, 16)])
+def test_profile_of_values_beyond_fp32_only_together(nx, ny):
+    """Four of 3e38 a row apart: no thread's own sum leaves FP32's range, that of the warp or block does."""
+    with flb.flb_create_ex(flb.config(nx, ny, 4, store="f32", pattern="aa")) as ctx:
+        n = relative_perturbation((4, ny, nx), seed=3, amp=0.02) / 19
+        n[3, 1, :8:2, 5] = 3e38
+        ctx.flb_set_populations(n)
+        n = ctx.flb_get_populations()
+        rho, j = ctx.flb_z_profile()
+    want_rho, want_j = reference(n, False)
+    assert np.isfinite(rho).all() and np.allclose(rho, want_rho, rtol=1e-12) and np.allclose(j, want_j, rtol=1e-12, atol=1e-13)
