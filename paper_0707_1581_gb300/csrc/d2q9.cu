@@ -87,6 +87,10 @@ constexpr int vec_width()
 // FP64 waits for its loads, but for AB steps without a force of 1.5 to 2 blocks per SM:
 // those kernels leave room for three blocks on an SM, so some SMs get three while others
 // hold one; the other FP64 kernels leave room for two.
+// AA even steps of more than two blocks per SM keep their loads in order: the compiler
+// spends six fewer FP64 instructions per thread on them and 76 registers (three blocks
+// per SM) instead of 82 (4096 x 2049, even and odd steps 1532 us, 1556 without); below,
+// the third block would crowd as above.
 //   FP64 AB  256 x 456 (228 blocks)  32.80 / - / 30.23 / 30.16; in graphs 30.75 / - / 30.40 / 31.09
 //            256 x 480 (240)         32.80 / - / 44.08 / 30.69; in graphs 30.78 / - / 43.07 / 32.28
 //            256 x 600 (300)         32.82 / - / 44.23 / 35.79;  256 x 612 (306)  47.13 / - / 44.26 / 44.00
@@ -96,7 +100,9 @@ StartPoint start_point(const BoxStep<S> &b, int64_t blocks, bool in_graph)   // 
     constexpr int64_t kSMs = 152;
     constexpr int64_t kL2 = 128000000;
     if (sizeof(S) == 8)
-        return LAYOUT == kAB && !FORCE && 2 * blocks > 3 * kSMs && blocks <= 2 * kSMs ? kUnchained : kAfterLoads;
+        return LAYOUT == kAB && !FORCE && 2 * blocks > 3 * kSMs && blocks <= 2 * kSMs ? kUnchained
+               : LAYOUT == kAAEven && blocks > 2 * kSMs                               ? kAfterLoadsInOrder
+                                                                                      : kAfterLoads;
     if (sizeof(S) == 2) return blocks <= kSMs ? kAfterLoads : blocks <= 2 * kSMs ? kBeforeStores : kAtStart;
     const bool in_l2 = (LAYOUT == kAB ? 2 : 1) * Q * b.plane * (int64_t)sizeof(S) <= kL2;
     // a graph's launches are close enough for a state in L2: 632 x 640 FP32 takes 5.82 us
@@ -117,6 +123,11 @@ cudaError_t step_vec(const BoxStep<S> &b, dim3 grid, dim3 block, const uint32_t 
     if constexpr (sizeof(S) < 8) {
         if (at == kBeforeStores)
             return launch_chained(k_stream_collide_vec<S, LAYOUT, NOISE, FORCE, V, kBeforeStores>, grid, block, st, b, p, t);
+    }
+    if constexpr (sizeof(S) == 8 && LAYOUT == kAAEven) {
+        if (at == kAfterLoadsInOrder)
+            return launch_chained(k_stream_collide_vec<S, LAYOUT, NOISE, FORCE, V, kAfterLoadsInOrder>, grid, block, st, b,
+                                  p, t);
     }
     if constexpr (sizeof(S) >= 4) {
         if (at == kUnchained) {

@@ -256,11 +256,19 @@ __global__ void __launch_bounds__(256) k_stream_collide(const BoxStep<S> B, cons
 // accesses.  The +-1 x-shift comes by warp shuffle from the neighbouring lane
 // (which owns the adjacent group whenever the group is not at a row end),
 // else by one scalar access; all lanes reach every shuffle.
-template <class S, int V>
+// IN_ORDER (FP64): the loads stay in the order of the source (see kAfterLoadsInOrder).
+template <class S, int V, bool IN_ORDER = false>
 __device__ __forceinline__ void load_vec2(const S *p, S (&out)[V])
 {
     using T = typename RawVec2<sizeof(S) * V>::T;
-    const T raw = *reinterpret_cast<const T *>(p);
+    T raw;
+    if constexpr (IN_ORDER)
+        asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(raw.x), "=r"(raw.y), "=r"(raw.z), "=r"(raw.w)
+                     : "l"(__cvta_generic_to_global(p))
+                     : "memory");
+    else
+        raw = *reinterpret_cast<const T *>(p);
     const S *e = reinterpret_cast<const S *>(&raw);
 #pragma unroll
     for (int v = 0; v < V; ++v) out[v] = e[v];
@@ -309,11 +317,11 @@ k_stream_collide_vec(const BoxStep<S> B, const uint32_t *step_ptr, uint32_t step
             slot = LAYOUT == kAB ? i : opposite(i);
         }
         const S *base = B.src + (int64_t)slot * B.plane + ro;
-        load_vec2<S, V>(FLB_GUARD_LD(B, base + x0, V), raw[i]);
+        load_vec2<S, V, START == kAfterLoadsInOrder>(FLB_GUARD_LD(B, base + x0, V), raw[i]);
         if (LAYOUT != kAAEven && cx > 0) edge[i] = load_ro(FLB_GUARD_LD(B, base + x_lload, 1));
         if (LAYOUT != kAAEven && cx < 0) edge[i] = load_ro(FLB_GUARD_LD(B, base + x_rload, 1));
     }
-    if constexpr (START == kAfterLoads) let_next_step_start();
+    if constexpr (START == kAfterLoads || START == kAfterLoadsInOrder) let_next_step_start();
     R f[V][Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {

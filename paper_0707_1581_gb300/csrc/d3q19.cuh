@@ -784,8 +784,9 @@ __device__ __forceinline__ void let_next_step_start() { asm volatile("griddepcon
 __device__ __forceinline__ void wait_for_previous_step() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Where a step kernel calls let_next_step_start (kUnchained: launched without
-// programmatic serialization, where that is the faster).
-enum StartPoint : int { kUnchained = -1, kAtStart = 0, kAfterLoads = 1, kBeforeStores = 2 };
+// programmatic serialization, where that is the faster; kAfterLoadsInOrder: as
+// kAfterLoads, with the loads in the order of the source).
+enum StartPoint : int { kUnchained = -1, kAtStart = 0, kAfterLoads = 1, kBeforeStores = 2, kAfterLoadsInOrder = 3 };
 
 // --------------------------------------------------------------------------
 // Where the canonical pre-collision population n_i(r, t) lives in device memory.

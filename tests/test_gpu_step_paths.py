@@ -238,3 +238,17 @@ def test_boxes_of_more_planes_or_rows_than_a_grid_dimension(nx, ny, nz, store):
             ctx.flb_step(3)
             got.append(ctx.flb_get_sites(sites))
     assert np.abs(got[0] - got[1]).max() <= TOLERANCE[store]
+
+
+@pytest.mark.parametrize("nx,ny", [(256, 608), (256, 610), (1000, 601)])
+@pytest.mark.parametrize("force,kT", [(0.0, 1e-4), (1e-5, 1e-4), (1e-5, 0.0)])
+def test_fp64_d2q9_steps_in_place_equal_the_one_site_kernel(nx, ny, force, kT):
+    """AA steps on either side of two blocks per SM against the one-site kernel: the same arithmetic, so FP64 bounds."""
+    cfg = box(nx, ny, 1, "f64", "aa", lattice="d2q9", kT=kT, force_amp=force)
+    got = []
+    for launch in ((2, 128, 2), (1, 128, 2)):
+        with flb.flb_create_ex(cfg) as ctx:
+            ctx.flb_set_launch(*launch)
+            ctx.flb_step(6)
+            got.append(ctx.flb_get_populations())
+    assert np.abs(got[0] - got[1]).max() <= TOLERANCE["f64"]
