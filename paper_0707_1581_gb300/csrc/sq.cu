@@ -684,7 +684,9 @@ __global__ void __launch_bounds__(256, 3) k_sq_lines(Cx<T> *X, int L, int64_t sl
                                                   SqRadices rd, SqShells sh, const uint16_t *__restrict__ tab, T inv_n,
                                                   int lmul)
 {
-    let_next_step_start();
+    // the FP64 transform ends with its z pass, which is not followed early (see k_sq_finish): 32^3, a step and a
+    // sample 121 us, 126 with an early start
+    if constexpr (!(ACC && sizeof(T) == 8)) let_next_step_start();
     wait_for_previous_step();
     const int W = 1 << lgW;
     extern __shared__ __align__(16) unsigned char sq_smem[];
