@@ -1919,7 +1919,7 @@ const char *flb_create_error(void)
 int flb_version(char *buf, int len)
 {
     if (!buf || len < 1) return FLB_EINVAL;
-    snprintf(buf, (size_t)len, "flb 0.2 (D3Q19 and D2Q9 fluctuating LB; sm_103a; CUDA %d)", CUDART_VERSION);
+    snprintf(buf, (size_t)len, "flb 0.3 (D3Q19 and D2Q9 fluctuating LB; sm_103a; CUDA %d)", CUDART_VERSION);
     return FLB_OK;
 }
 

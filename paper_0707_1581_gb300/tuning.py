@@ -4,9 +4,10 @@
 on a hit it applies the recorded streaming pattern and launch shape
 (flb_set_pattern, flb_set_launch), on a miss it runs flb_autotune(_ex) and
 records the result.  The key holds the lattice, the storage format, every
-box's size, whether the pattern was tuned, the GPU's name and the library
-version; the choice is a pure function of those (the timings that produced it
-are not repeated).  Host logic only -- the tuning itself runs in libflb.so.
+box's size, what else selects a kernel (thermal noise, undamped kinetic modes,
+a body force), whether the pattern was tuned, the GPU's name and the library
+version, which changes with the meaning of a shape; the choice is a pure
+function of those (the timings that produced it are not repeated).  Host logic only -- the tuning itself runs in libflb.so.
 """
 from __future__ import annotations
 
@@ -19,7 +20,11 @@ from . import flb
 def tuning_key(ctx, tune_pattern: bool, device: str) -> str:
     boxes = [[c.nx, c.ny, c.nz] for c in ctx.cfgs]
     c0 = ctx.cfgs[0]
+    def some(option: str) -> bool:
+        return any(getattr(c, option, 0.0) != 0.0 for c in ctx.cfgs)
+
     return json.dumps({"lattice": int(c0.lattice), "store": int(c0.store),
+                       "kernel": [some("kT"), some("gamma_ghost"), some("force_amp")],
                        "pattern": "tuned" if tune_pattern else int(c0.pattern),
                        "boxes": boxes, "device": device, "library": flb.flb_version()}, sort_keys=True)
 

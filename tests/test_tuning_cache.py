@@ -66,3 +66,17 @@ def test_key_separates_boxes_formats_devices_and_pattern_tuning(monkeypatch):
             tuning.tuning_key(FakeContext([Cfg(64, 64, 64, store=2)]), False, "A"),
             tuning.tuning_key(FakeContext([Cfg(64, 64, 1, lattice=1)]), False, "A")}
     assert len(keys) == 6
+
+
+def test_key_separates_what_selects_another_kernel(monkeypatch):
+    """Thermal noise, undamped kinetic modes and a body force, in any box; not their values."""
+    monkeypatch.setattr(flb, "flb_version", lambda: "flb test")
+
+    def key(*boxes):
+        return tuning.tuning_key(FakeContext([flb.config(16, 16, 16, **kw) for kw in boxes]), False, "A")
+
+    plain = dict(kT=0.0, gamma_ghost=0.0, force_amp=0.0)
+    options = [plain, dict(plain, kT=1e-4), dict(plain, gamma_ghost=0.1), dict(plain, force_amp=1e-5)]
+    assert len({key(o) for o in options}) == 4
+    assert len({key(plain, o) for o in options}) == 4
+    assert key(dict(plain, kT=1e-4)) == key(dict(plain, kT=2e-4))
