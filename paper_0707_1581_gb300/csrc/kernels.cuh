@@ -710,18 +710,22 @@ struct BatchParams {
 //   V = 2, 24 boxes of 50^3: FP16 AB 69.6 (2) 63.5 (3) 57.3 (4), AA 61.4 (3) 62.0 (4);
 //     bfloat16 AB 64.4 / 58.0, AA 62.9 / 62.0; stochastic AB 78.8 / 79.5, AA 82.3 / 83.8;
 //     FP32 AB 86.6 (2) 76.5 (3) 70.1 (4), AA 77.2 (3) 79.1 (4)
+//   V = 2, 16 boxes of 24^3, less than a wave: FP16 AB 5.90 (3) 6.25 (4), AA 6.04 / 7.05;
+//     11 boxes of 32^3, whose rows tile the warps: FP32 AB 8.72 / 10.0, FP16 AA 8.51 / 9.14
 //   V = 1, 8 boxes of 65^3, whose threads hold their normals over the wait (82 to 90
 //     registers when left free): stochastic AB 76.0 (2) 74.3 (4) 71.2 (5); FP16 AB 61.6 /
 //     58.9 / 56.5; FP32 AB 60.7 (3) 54.1 (5); AA 75.5 with 5, 74.5 free (stochastic),
 //     86.6 / 59.0 (FP16), where five blocks spill
+// So AB steps of two sites take four blocks, but three in launches of a wave or less and
+// in FP32 where every box's rows tile the warps (step_batch in step_impl.cuh).
 template <class S, int LAYOUT, int V>
 constexpr int kBatchMinBlocks = sizeof(S) == 8 ? 1
                                 : V == 4       ? kMinBlocks<S, V, kEdges>
                                 : V == 1       ? (LAYOUT == kAB ? 5 : 1)
-                                : Storage<S>::stochastic || (sizeof(S) == 4 && LAYOUT != kAB) ? 3 : 4;
+                                : Storage<S>::stochastic || LAYOUT != kAB ? 3 : 4;
 
-template <class S, int LAYOUT, int NOISE, bool FORCE, int V>
-__global__ void __launch_bounds__(256, kBatchMinBlocks<S, LAYOUT, V>)
+template <class S, int LAYOUT, int NOISE, bool FORCE, int V, int MIN_BLOCKS = kBatchMinBlocks<S, LAYOUT, V>>
+__global__ void __launch_bounds__(256, MIN_BLOCKS)
 k_stream_collide_batch(const __grid_constant__ BatchParams<S> P, const uint32_t *step_ptr, uint32_t step)
 {
     if constexpr (kStart<S, V> == kAtStart) let_next_step_start();

@@ -53,6 +53,14 @@ cudaError_t step_batch(const BatchParams<S> &P, int total_blocks, const Launch &
                        uint32_t step, cudaStream_t st)
 {
     const dim3 block(L.bx * L.by);
+    if constexpr (kBatchMinBlocks<S, LAYOUT, V> == 4) {
+        // three blocks of 256 threads per SM instead of four (see kBatchMinBlocks)
+        bool tiled = sizeof(S) == 4;
+        for (int k = 0; k < P.nboxes; ++k) tiled = tiled && P.boxes[k].warprow;
+        if (tiled || (int64_t)total_blocks * (int64_t)block.x <= 4 * 152 * 256)
+            return launch_chained(k_stream_collide_batch<S, LAYOUT, NOISE, FORCE, V, 3>, dim3(total_blocks), block, st, P,
+                                  step_ptr, step);
+    }
     return launch_chained(k_stream_collide_batch<S, LAYOUT, NOISE, FORCE, V>, dim3(total_blocks), block, st, P,
                           step_ptr, step);
 }
