@@ -37,8 +37,10 @@ struct Launch {
     bool edgerow = false;   // blocks of one row each, scalar accesses at row and warp ends
 };
 
-// Gives the pages of a host array that is about to be overwritten (host_mem.cu).
-void prefault(void *p, size_t bytes);
+// Gives the pages of a host array that is about to be overwritten, from `least` bytes on;
+// true if they were not there (host_mem.cu).
+enum PageLook { kLookAtLast, kLookAtAll };   // which pages it looks at to know
+bool prefault(void *p, size_t bytes, PageLook look, size_t least = size_t(1) << 20);
 
 // Launches a kernel of the step or sampling chain with programmatic stream
 // serialization: its blocks may start once every block of the kernel before it has
