@@ -257,7 +257,9 @@ inline int profile_chunks(int64_t M, int units, int nq)
 
 // The means of the units of one pass over a box (d2: D2Q9): part is scratch of nq
 // nsum chunks doubles, out receives 4 n doubles.  Units of fewer than 2048 elements
-// are summed by one warp each.
+// are summed by one warp each (D2Q9 FP32 1500 x 1200: 48 us per call, 58 with blocks),
+// but from 1024 on by blocks where there are too few units to fill the SMs with warps
+// (48 x 40 x 36: 24.2 us, 26.2 with warps).
 template <class S>
 cudaError_t launch_profile(const S *buf, int64_t plane, int layout, int64_t M, int units, const profile::Pass &P, bool d2,
                            double rho0, double *part, double *out, cudaStream_t st)
@@ -265,7 +267,7 @@ cudaError_t launch_profile(const S *buf, int64_t plane, int layout, int64_t M, i
     const int nq = d2 ? 9 : Q, chunks = profile_chunks(M, units, nq);
     const int64_t items = (int64_t)P.nsum * nq * chunks;
     constexpr int T = profile::kThreads;
-    if (M < 2048)
+    if (M < 1024 || (M < 2048 && items > 1216))
         profile::k_unit_sums<S, 32><<<(unsigned)((items + T / 32 - 1) / (T / 32)), T, 0, st>>>(buf, plane, M, units, P,
                                                                                                items, chunks, part);
     else

@@ -139,3 +139,15 @@ def test_profile_of_values_beyond_fp32_only_together(nx, ny):
         rho, j = ctx.flb_z_profile()
     want_rho, want_j = reference(n, False)
     assert np.isfinite(rho).all() and np.allclose(rho, want_rho, rtol=1e-12) and np.allclose(j, want_j, rtol=1e-12, atol=1e-13)
+
+
+@pytest.mark.parametrize("store", ["f64", "f32", "bf16sr"])
+def test_profile_on_either_side_of_warps_and_blocks(store):
+    """Planes of 1023, 1024, 2025 and 2048 elements; 64 and 65 planes (1216 and 1235 sums)."""
+    for nx, ny, nz in ((33, 31, 20), (32, 32, 64), (32, 32, 65), (45, 45, 8), (64, 32, 3)):
+        with flb.flb_create_ex(flb.config(nx, ny, nz, kT=1e-3, gamma_shear=0.3, seed=2, store=store)) as ctx:
+            ctx.flb_step(2)
+            rho, j = ctx.flb_z_profile()
+            want_rho, want_j = reference(ctx.flb_get_populations(), False)
+        # as in the first test
+        assert np.abs(rho - want_rho).max() <= 2e-14 and np.abs(j - want_j).max() <= 2e-14, (nx, ny, nz)
