@@ -358,7 +358,7 @@ __device__ __forceinline__ void forward_modes(const R (&f)[Q], R (&m)[Q])
 // Two orders of the arithmetic.  collide (FP32, one site or a pair) takes about
 // 180 operations per site with gamma_ghost = 0.  collide64 takes about 150: FP64
 // kernels are bound by the FP64 unit (64 cycles per warp instruction on each SM
-// quarter), and 128^3 takes 677 us per step with it against 772.  FP32 keeps its
+// quarter), and 128^3 takes 672 us per step with it against 772.  FP32 keeps its
 // order although collide64's would give the 16-bit kernels 4-8 %: a stored value's
 // rounding to 16 bits follows the last FP32 bit, so another order gives another
 // (equally good) run -- the total momentum of a bfloat16 box differs in its second
@@ -774,7 +774,7 @@ __device__ __forceinline__ bool span_ok(const S *base, int64_t plane, const S *p
 // --------------------------------------------------------------------------
 // Chained steps.  The step kernels are launched with programmatic stream
 // serialization: a step's blocks are scheduled as soon as every block of the
-// step before has started (let_next_step_start), and do what needs no stored
+// step before has called let_next_step_start, and do what needs no stored
 // state -- index arithmetic, and in the small-box kernels the Gaussian numbers
 // -- before wait_for_previous_step, which returns when the whole step before has
 // finished and its writes are visible.  Every block of every step kernel

@@ -178,8 +178,8 @@ __device__ __forceinline__ void stats_pass(const S *__restrict__ buf, int64_t pl
 {
     // Per site everything runs in the compute type R on the stored deviations
     // n_i - rho0 a_i.  Each lane keeps R partial sums of about 16 sites; at
-    // warp-uniform points a warp adds its lanes' partials (fixed butterfly
-    // order) and lane 0 adds the result to the warp's FP64 row in shared
+    // warp-uniform points a warp adds its lanes' partials (warp_sums, a fixed
+    // butterfly order) and lane k adds sum k to the warp's FP64 row in shared
     // memory, so FP64 arithmetic and the FP64 registers stay off the per-site
     // path.  Every order is fixed: the result is bitwise reproducible.
     let_next_step_start();   // the pass over the partial sums (started as usual: it reads by the read-only path)

@@ -193,7 +193,7 @@ __device__ __forceinline__ void stage(const Cx<T> *__restrict__ src, Cx<T> *__re
 // and output.  The inputs are folded in place first (the stage's source is not
 // needed afterwards); then a thread takes kQ output pairs of one butterfly, so that
 // a loaded A_r, B_r serves all of them.  140 x 491 x 40 FP32, the sample's S(q):
-// 4320 us with two products per r and output, KSQ491 now.
+// 4330 us with two products per r and output, 194 now.
 template <class T>
 __device__ void stage_generic(Cx<T> *src, Cx<T> *__restrict__ dst, const Cx<T> *tw, int L, int Ls, int Ns, int nl, int R)
 {
